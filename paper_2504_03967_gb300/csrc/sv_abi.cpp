@@ -285,6 +285,7 @@ int sv_free(sv_handle h) {
     if (h->perm_tmp.ptr) cudaFree(h->perm_tmp.ptr);
     if (h->aux.ptr) cudaFree(h->aux.ptr);
     if (h->lcdf.ptr) cudaFree(h->lcdf.ptr);
+    if (h->fine.ptr) cudaFree(h->fine.ptr);
     delete h->plans;
     if (h->host_pin.ptr) cudaFreeHost(h->host_pin.ptr);
     for (cudaEvent_t e : h->ev_pool) cudaEventDestroy(e);

@@ -295,6 +295,7 @@ struct sv_state {
     sv::Scratch perm_tmp;    // device scratch of the permuted read-outs
     sv::Scratch aux;         // device scratch of the QCrank read-out (shots, counters, pixels)
     sv::Scratch lcdf;        // device scratch of the logical-order block CDF of a relabelled state
+    sv::Scratch fine;        // device scratch of the samplers' CDF table (many shots)
     long long pending_basis; // >= 0: sv_init_basis(x) not written yet (the next apply's first pass or any other
                              // use of the state writes it)
     sv::PlanCache* plans;    // recent plans of this handle (sv_apply_circuit)

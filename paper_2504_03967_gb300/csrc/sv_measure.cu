@@ -79,10 +79,13 @@ __device__ __forceinline__ FF ff_allreduce(FF a) {
 // gives the lane's total and its sums over j with bit b set (57 double-float
 // additions for 32 amplitudes), and one reduce-scatter across the warp sums
 // the 11 per-lane values (total, total where lane bit b is set, the 5 j-bit
-// sums): each of the first four exchange steps halves the values a lane
-// keeps, so lane 2e (e < 11) ends with value e summed over all 32 lanes.
+// sums) and, in slots the exchange carries anyway, the totals of the block's
+// first three quarters (256 amplitudes each, for the sampler): each of the
+// first four exchange steps halves the values a lane keeps, so lane 2e
+// (e < 14) ends with value e summed over all 32 lanes.
 __device__ __forceinline__ void block_stats_c64_full(const float2* __restrict__ psi, uint64_t wid, int lane,
-                                                     double* __restrict__ tot, double* __restrict__ bits) {
+                                                     double* __restrict__ tot, double* __restrict__ bits,
+                                                     double* __restrict__ quart) {
     const uint64_t b0 = wid << 10;
     FF p[32];
 #pragma unroll
@@ -108,12 +111,16 @@ __device__ __forceinline__ void block_stats_c64_full(const float2* __restrict__ 
             ff_add(t, p[2 * i + 1].hi, p[2 * i + 1].lo);
             p[i] = t;
         }
+        if (lev == 2) {  // p[q]: this lane's sum over quarter q
+#pragma unroll
+            for (int q = 0; q < 3; ++q) e[11 + q] = p[q];
+        }
     }
     e[0] = p[0];
 #pragma unroll
     for (int b = 0; b < 5; ++b) e[1 + b] = ((lane >> b) & 1) ? p[0] : FF{0.f, 0.f};
 #pragma unroll
-    for (int k = 11; k < 16; ++k) e[k] = FF{0.f, 0.f};
+    for (int k = 14; k < 16; ++k) e[k] = FF{0.f, 0.f};
 #pragma unroll
     for (int st = 0; st < 4; ++st) {  // lane bits 4, 3, 2, 1
         const int h = 8 >> st, mask = 16 >> st;
@@ -130,16 +137,18 @@ __device__ __forceinline__ void block_stats_c64_full(const float2* __restrict__ 
     }
     ff_add(e[0], __shfl_xor_sync(0xffffffffu, e[0].hi, 1), __shfl_xor_sync(0xffffffffu, e[0].lo, 1));
     const int idx = ((lane >> 4) & 1) * 8 + ((lane >> 3) & 1) * 4 + ((lane >> 2) & 1) * 2 + ((lane >> 1) & 1);
-    if (!(lane & 1) && idx < 11) {
+    if (!(lane & 1) && idx < 14) {
         const double val = ff_val(e[0]);
         if (idx == 0) tot[wid] = val;
-        else bits[wid * 10 + (idx - 1)] = val;  // 1..5: lane bits 0..4; 6..10: j bits = index bits 5..9
+        else if (idx < 11) bits[wid * 10 + (idx - 1)] = val;  // 1..5: lane bits 0..4; 6..10: j bits = index bits 5..9
+        else if (quart) quart[wid * 4 + (idx - 11)] = val;
     }
 }
 
 template <typename V>
 __global__ void __launch_bounds__(256) k_block_stats(const V* __restrict__ psi, int blog, uint64_t nblocks,
-                                                     double* __restrict__ tot, double* __restrict__ bits) {
+                                                     double* __restrict__ tot, double* __restrict__ bits,
+                                                     double* __restrict__ quart) {
     const int lane = threadIdx.x & 31;
     const uint64_t wid = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (wid >= nblocks) return;
@@ -148,7 +157,7 @@ __global__ void __launch_bounds__(256) k_block_stats(const V* __restrict__ psi, 
     const int jn = len >= 32 ? len / 32 : 1;
     if constexpr (sizeof(V) == 8) {
         if (bits && blog == 10) {
-            block_stats_c64_full((const float2*)psi, wid, lane, tot, bits);
+            block_stats_c64_full((const float2*)psi, wid, lane, tot, bits, quart);
             return;
         }
         FF acc = {0.f, 0.f}, ab[5];
@@ -254,8 +263,9 @@ __global__ void k_expz_final(const double* __restrict__ part, int n, double* __r
 }
 
 // ---- inclusive scan of doubles -------------------------------------------
-// One CTA of 1024 threads scans CH = 8192 consecutive values in place
-// (8 per thread sequentially, then a CTA scan of the thread totals), adding
+// One CTA of 1024 threads scans CH = 8192 consecutive values of a into out
+// (which may be a; 8 per thread sequentially, then a CTA scan of the thread
+// totals), adding
 // "offset" (an exclusive prefix from the chunk scan, or 0).
 constexpr int kScanT = 1024;
 constexpr int kScanPer = 8;
@@ -290,7 +300,7 @@ __device__ double cta_exclusive_scan(double v, double* total) {
     return excl;
 }
 
-__global__ void __launch_bounds__(kScanT) k_scan_chunks(double* __restrict__ a, uint64_t len,
+__global__ void __launch_bounds__(kScanT) k_scan_chunks(const double* a, double* out, uint64_t len,
                                                         const double* __restrict__ offsets) {
     const uint64_t c0 = (uint64_t)blockIdx.x * kScanCh;
     const uint64_t i0 = c0 + (uint64_t)threadIdx.x * kScanPer;
@@ -305,7 +315,7 @@ __global__ void __launch_bounds__(kScanT) k_scan_chunks(double* __restrict__ a, 
     const double ex = cta_exclusive_scan(s, nullptr) + (offsets ? offsets[blockIdx.x] : 0.0);
 #pragma unroll
     for (int j = 0; j < kScanPer; ++j)
-        if (i0 + j < len) a[i0 + j] = loc[j] + ex;
+        if (i0 + j < len) out[i0 + j] = loc[j] + ex;
 }
 
 __global__ void __launch_bounds__(kScanT) k_chunk_totals(const double* __restrict__ a, uint64_t len,
@@ -451,14 +461,183 @@ __global__ void __launch_bounds__(256) k_block_tot_logical(const V* __restrict__
     }
 }
 
-// ---- sampler: one warp per shot ------------------------------------------
+// ---- sampler --------------------------------------------------------------
+// Outcome = min{x : C_x > t}, t = u S.  Three ways to find x, the same answer:
+//
+//  * warp_sample: one warp per shot, the rule itself.  A 32-way search of the
+//    block CDF, then a rescan of the chosen block 32 amplitudes at a time (a
+//    coalesced load, a warp scan on top of the running CDF, a ballot).
+//  * warp_sample_quarter (complex64, 1024-amplitude blocks with quarter
+//    totals): the quarter totals leave 256 of the 1024 amplitudes to read,
+//    and one warp scan finds x among them.
+//  * k_sample_dense (about as many shots as amplitudes, or more): a table of
+//    C_x for every x and a guide into it, one thread per shot.
+//
+// The two short cuts add the probabilities in another order than warp_sample,
+// which moves a C_x by some 10^-15 S.  They therefore take an x only when t is
+// clear of both its ends, C_{x-1} < t - d and C_x > t + d with d = kClear S
+// far above that; otherwise (about one shot in 10^11 / 2^n) the warp falls
+// back to warp_sample, so every outcome is the one warp_sample gives.
+constexpr double kClear = 1e-12;
+
+// First block j with cdf[j] > t (the last block if rounding leaves none): a
+// 32-way search, each lane testing one of 32 evenly spaced entries of
+// [lo, hi), so 2^18 blocks take four steps; the answer stays in [lo, hi) and
+// lane 31 always tests hi - 1.
+__device__ __forceinline__ uint64_t warp_find_block(const double* __restrict__ cdf, uint64_t nblocks, double t,
+                                                    int lane) {
+    uint64_t lo = 0, hi = nblocks;
+    while (hi - lo > 1) {
+        const uint64_t step = (hi - lo + 31) >> 5;
+        const uint64_t at = min(lo + (uint64_t)(lane + 1) * step, hi) - 1;
+        const unsigned yes = __ballot_sync(0xffffffffu, at == nblocks - 1 || cdf[at] > t);
+        const int f = __ffs(yes) - 1;
+        const uint64_t at_f = __shfl_sync(0xffffffffu, at, f);
+        const uint64_t at_p = __shfl_sync(0xffffffffu, at, f > 0 ? f - 1 : 0);
+        hi = at_f + 1;
+        if (f > 0) lo = at_p + 1;
+    }
+    return lo;
+}
+
+// Rescan of block j.  complex64: |a|^2 as an exact float pair and the scan in
+// double-float (about 48 bits; no FP64 instruction in the loop) when the
+// state's total S lies well inside FP32's range; complex128, or a far from
+// normalised state: FP64.  The first lane whose CDF exceeds t (and whose
+// probability is not zero) is the outcome.
+template <typename V, class Amp>
+__device__ __forceinline__ uint64_t warp_sample(const Amp& amp, int blog, const double* __restrict__ cdf, uint64_t j,
+                                                double S, double t, int lane) {
+    const uint64_t len = 1ull << blog;
+    const double before = j ? cdf[j - 1] : 0.0;
+    const uint64_t b0 = j << blog;
+    uint64_t pick = UINT64_MAX, last_nz = b0;
+    if constexpr (sizeof(V) == 8) {
+        if (S > 1e-20 && S < 1e20) {
+            const FF tf = ff_of(t);
+            FF base = ff_of(before);
+            for (uint64_t c = 0; c < len; c += 32) {
+                const bool valid = c + lane < len;
+                FF p = {0.f, 0.f};
+                if (valid) p = ff_prob(amp(b0 + c + lane));
+                FF inc = p;
+#pragma unroll
+                for (int sh = 1; sh < 32; sh <<= 1) {
+                    const float h = __shfl_up_sync(0xffffffffu, inc.hi, sh);
+                    const float l = __shfl_up_sync(0xffffffffu, inc.lo, sh);
+                    if (lane >= sh) ff_add(inc, h, l);
+                }
+                FF cum = base;
+                ff_add(cum, inc.hi, inc.lo);
+                const float above = (cum.hi - tf.hi) + (cum.lo - tf.lo);  // sign of cum - t
+                const unsigned hit = __ballot_sync(0xffffffffu, valid && p.hi > 0.f && above > 0.f);
+                if (hit) {
+                    pick = b0 + c + (uint64_t)(__ffs(hit) - 1);
+                    break;
+                }
+                const unsigned nz = __ballot_sync(0xffffffffu, p.hi > 0.f);
+                if (nz) last_nz = b0 + c + (uint64_t)(31 - __clz(nz));
+                ff_add(base, __shfl_sync(0xffffffffu, inc.hi, 31), __shfl_sync(0xffffffffu, inc.lo, 31));
+            }
+            return pick == UINT64_MAX ? last_nz : pick;
+        }
+    }
+    double base = before;
+    for (uint64_t c = 0; c < len; c += 32) {
+        const bool valid = c + lane < len;
+        const double p = valid ? prob(amp(b0 + c + lane)) : 0.0;
+        double inc = p;
+#pragma unroll
+        for (int sh = 1; sh < 32; sh <<= 1) {
+            const double y = __shfl_up_sync(0xffffffffu, inc, sh);
+            if (lane >= sh) inc += y;
+        }
+        const unsigned hit = __ballot_sync(0xffffffffu, valid && p > 0.0 && base + inc > t);
+        if (hit) {
+            pick = b0 + c + (uint64_t)(__ffs(hit) - 1);
+            break;
+        }
+        const unsigned nz = __ballot_sync(0xffffffffu, p > 0.0);
+        if (nz) last_nz = b0 + c + (uint64_t)(31 - __clz(nz));  // fallback when rounding leaves no x above t
+        base += __shfl_sync(0xffffffffu, inc, 31);
+    }
+    return pick == UINT64_MAX ? last_nz : pick;
+}
+
+// Block j (1024 amplitudes of complex64) with its quarter totals: the quarter
+// from its totals, then lane l adds the quarter's amplitudes 8 l .. 8 l + 7 (64
+// contiguous bytes, 2 KB per warp), one warp scan of the lane sums picks the
+// lane, and its eight probabilities, sent to all lanes, give x.  All compares
+// are against t minus the quarter's start, in double-float (a float pair holds
+// 48 bits of a value of at most S, far below kClear S).  UINT64_MAX: t is not
+// clear of the neighbouring outcomes.  Bound by the 2 KB read per shot; with
+// the whole block (8 KB, 32 dependent scan steps of which half are taken on
+// average) 10^5 shots of a 28-qubit state took 339 us.
+__device__ __forceinline__ uint64_t warp_sample_quarter(const float2* __restrict__ psi, const double* __restrict__ cdf,
+                                                        const double* __restrict__ quart, uint64_t j, double S, double t,
+                                                        int lane) {
+    const double before = j ? cdf[j - 1] : 0.0;
+    double r = t - before;  // what is left of t inside the block
+    int q = 0;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {  // (uniform across the warp)
+        const double w = quart[j * 4 + k];
+        if (q == k && r >= w) {
+            r -= w;
+            q = k + 1;
+        }
+    }
+    const float4* src = (const float4*)(psi + (j << 10) + (q << 8)) + 4 * lane;
+    FF p[8], sum{0.f, 0.f};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const float4 v = src[i];
+        p[2 * i] = ff_prob(make_float2(v.x, v.y));
+        p[2 * i + 1] = ff_prob(make_float2(v.z, v.w));
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) ff_add(sum, p[i].hi, p[i].lo);
+    FF inc = sum;
+#pragma unroll
+    for (int sh = 1; sh < 32; sh <<= 1) {
+        const float h = __shfl_up_sync(0xffffffffu, inc.hi, sh);
+        const float l = __shfl_up_sync(0xffffffffu, inc.lo, sh);
+        if (lane >= sh) ff_add(inc, h, l);
+    }
+    const FF rf = ff_of(r);
+    const unsigned over = __ballot_sync(0xffffffffu, (inc.hi - rf.hi) + (inc.lo - rf.lo) > 0.f);
+    if (!over) return UINT64_MAX;
+    const int f = __ffs(over) - 1;
+    FF cum{0.f, 0.f};
+    if (f) {
+        cum.hi = __shfl_sync(0xffffffffu, inc.hi, f - 1);
+        cum.lo = __shfl_sync(0xffffffffu, inc.lo, f - 1);
+    }
+    const float d = (float)(kClear * S);
+    float prev = (cum.hi - rf.hi) + (cum.lo - rf.lo);  // C_{x-1} - t
+    int at = 8;
+    bool clear = false;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        ff_add(cum, __shfl_sync(0xffffffffu, p[i].hi, f), __shfl_sync(0xffffffffu, p[i].lo, f));
+        const float cur = (cum.hi - rf.hi) + (cum.lo - rf.lo);
+        if (at == 8 && cur > 0.f) {
+            at = i;
+            clear = prev < -d && cur > d;
+        }
+        prev = cur;
+    }
+    return clear ? (j << 10) + (uint64_t)(q << 8) + 8 * f + at : UINT64_MAX;
+}
+
 // PERM (a relabelled state): cdf is the block CDF in LOGICAL order (from
 // k_block_tot_logical) and the chosen block is rescanned in logical order,
 // amplitude x read at its physical index; the outcome is the logical x.
+// quart: quarter totals of the blocks (complex64, blog = 10), or nullptr.
 template <typename V, bool PERM>
-__global__ void __launch_bounds__(256) k_sample(const V* __restrict__ psi, int n, int blog,
-                                                const double* __restrict__ cdf, uint64_t nblocks,
-                                                uint64_t shots, uint64_t seed, const double* __restrict__ u_in,
+__global__ void __launch_bounds__(256) k_sample(const V* __restrict__ psi, int blog, const double* __restrict__ cdf,
+                                                uint64_t nblocks, const double* __restrict__ quart, uint64_t shots,
+                                                uint64_t seed, const double* __restrict__ u_in,
                                                 uint64_t* __restrict__ out, const QubitMap map) {
     __shared__ uint64_t qt[PERM ? 5 : 1][256];
     if constexpr (PERM) {
@@ -472,88 +651,143 @@ __global__ void __launch_bounds__(256) k_sample(const V* __restrict__ psi, int n
     const int lane = threadIdx.x & 31;
     const uint64_t warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
     const double S = cdf[nblocks - 1];
-    const uint64_t len = 1ull << blog;
+    const bool short_cut = quart && S > 1e-20 && S < 1e20;
     for (uint64_t s = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; s < shots; s += warps) {
         const double u = u_in ? u_in[s] : philox_uniform(seed, s);
         const double t = u * S;
-        // first block j with cdf[j] > t (the last block if rounding leaves
-        // none): a 32-way search, each lane testing one of 32 evenly spaced
-        // entries of [lo, hi), so 2^18 blocks take four steps; the answer
-        // stays in [lo, hi) and lane 31 always tests hi - 1
-        uint64_t lo = 0, hi = nblocks;
-        while (hi - lo > 1) {
-            const uint64_t step = (hi - lo + 31) >> 5;
-            const uint64_t at = min(lo + (uint64_t)(lane + 1) * step, hi) - 1;
-            const unsigned yes = __ballot_sync(0xffffffffu, at == nblocks - 1 || cdf[at] > t);
-            const int f = __ffs(yes) - 1;
-            const uint64_t at_f = __shfl_sync(0xffffffffu, at, f);
-            const uint64_t at_p = __shfl_sync(0xffffffffu, at, f > 0 ? f - 1 : 0);
-            hi = at_f + 1;
-            if (f > 0) lo = at_p + 1;
-        }
-        const uint64_t j = lo;
-        const double before = j ? cdf[j - 1] : 0.0;
-        const uint64_t b0 = j << blog;
-        // rescan the block 32 amplitudes at a time (one coalesced load per
-        // step): a warp scan of the step's probabilities on top of the
-        // running CDF, and the first lane whose CDF exceeds t (and whose
-        // probability is not zero) is the outcome.  complex64: |a|^2 as an
-        // exact float pair and the scan in double-float (about 48 bits; no
-        // FP64 instruction in the loop) when the state's total lies well
-        // inside FP32's range; complex128, or a far from normalised state:
-        // FP64.
-        uint64_t pick = UINT64_MAX, last_nz = b0;
-        if constexpr (sizeof(V) == 8) {
-            if (S > 1e-20 && S < 1e20) {
-                const FF tf = ff_of(t);
-                FF base = ff_of(before);
-                for (uint64_t c = 0; c < len; c += 32) {
-                    const bool valid = c + lane < len;
-                    FF p = {0.f, 0.f};
-                    if (valid) p = ff_prob(amp(b0 + c + lane));
-                    FF inc = p;
+        const uint64_t j = warp_find_block(cdf, nblocks, t, lane);
+        uint64_t x = UINT64_MAX;
+        if constexpr (sizeof(V) == 8 && !PERM)
+            if (short_cut) x = warp_sample_quarter((const float2*)psi, cdf, quart, j, S, t, lane);
+        if (x == UINT64_MAX) x = warp_sample<V>(amp, blog, cdf, j, S, t, lane);
+        if (lane == 0) out[s] = x;
+    }
+}
+
+// ---- many shots: a table of the CDF ------------------------------------------
+// fine[x] = C_x for every amplitude (one warp per 32-amplitude block of the
+// block CDF, FP64) ...
+template <typename V, bool PERM>
+__global__ void __launch_bounds__(256) k_fine_cdf(const V* __restrict__ psi, const double* __restrict__ cdf,
+                                                  uint64_t nblocks, double* __restrict__ fine, const QubitMap map) {
+    __shared__ uint64_t qt[PERM ? 5 : 1][256];
+    if constexpr (PERM) {
+        build_byte_tables(qt, map);
+        __syncthreads();
+    }
+    const int lane = threadIdx.x & 31;
+    const uint64_t warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
+    for (uint64_t j = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; j < nblocks; j += warps) {
+        const uint64_t x = (j << 5) + lane;
+        double inc;
+        if constexpr (PERM) inc = prob(psi[phys_index(qt, x)]);
+        else inc = prob(psi[x]);
 #pragma unroll
-                    for (int sh = 1; sh < 32; sh <<= 1) {
-                        const float h = __shfl_up_sync(0xffffffffu, inc.hi, sh);
-                        const float l = __shfl_up_sync(0xffffffffu, inc.lo, sh);
-                        if (lane >= sh) ff_add(inc, h, l);
-                    }
-                    FF cum = base;
-                    ff_add(cum, inc.hi, inc.lo);
-                    const float above = (cum.hi - tf.hi) + (cum.lo - tf.lo);  // sign of cum - t
-                    const unsigned hit = __ballot_sync(0xffffffffu, valid && p.hi > 0.f && above > 0.f);
-                    if (hit) {
-                        pick = b0 + c + (uint64_t)(__ffs(hit) - 1);
-                        break;
-                    }
-                    const unsigned nz = __ballot_sync(0xffffffffu, p.hi > 0.f);
-                    if (nz) last_nz = b0 + c + (uint64_t)(31 - __clz(nz));
-                    ff_add(base, __shfl_sync(0xffffffffu, inc.hi, 31), __shfl_sync(0xffffffffu, inc.lo, 31));
-                }
-                if (lane == 0) out[s] = pick == UINT64_MAX ? last_nz : pick;
+        for (int sh = 1; sh < 32; sh <<= 1) {
+            const double y = __shfl_up_sync(0xffffffffu, inc, sh);
+            if (lane >= sh) inc += y;
+        }
+        fine[x] = (j ? cdf[j - 1] : 0.0) + inc;
+    }
+}
+// ... and guide[i] = first x with C_x > (i / N) S, i = 0..N (at most N - 1),
+// so that a shot with u in [i, i + 1) / N ends between guide[i] and
+// guide[i + 1]: about one table entry to read instead of a search of all.
+__global__ void __launch_bounds__(256) k_guide(const double* __restrict__ fine, uint32_t N, uint32_t* __restrict__ guide) {
+    const double step = fine[N - 1] / (double)N;  // (N is a power of two)
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i <= N; i += gridDim.x * blockDim.x) {
+        const double t = (double)i * step;
+        uint32_t lo = 0, hi = N - 1;
+        while (lo < hi) {
+            const uint32_t mid = (lo + hi) >> 1;
+            if (fine[mid] > t) hi = mid;
+            else lo = mid + 1;
+        }
+        guide[i] = lo;
+    }
+}
+
+// One thread per four shots (one Philox block): three random 32-byte sectors
+// of L2 per shot (guide, table, table) against a warp's search and rescan of
+// 32 amplitudes.  QCrank read-out of 2^20 amplitudes, 4.9 10^7 shots: one warp
+// per shot took 41.4 ms.
+template <typename V, bool PERM>
+__global__ void __launch_bounds__(256) k_sample_dense(const V* __restrict__ psi, const double* __restrict__ cdf,
+                                                      uint64_t nblocks, const double* __restrict__ fine,
+                                                      const uint32_t* __restrict__ guide, uint64_t shots, uint64_t seed,
+                                                      const double* __restrict__ u_in, uint64_t* __restrict__ out,
+                                                      const QubitMap map) {
+    __shared__ uint64_t qt[PERM ? 5 : 1][256];
+    if constexpr (PERM) {
+        build_byte_tables(qt, map);
+        __syncthreads();
+    }
+    auto amp = [&](uint64_t x) -> V {
+        if constexpr (PERM) return psi[phys_index(qt, x)];
+        else return psi[x];
+    };
+    const int lane = threadIdx.x & 31;
+    const double S = cdf[nblocks - 1], d = kClear * S, scale = (double)(nblocks << 5);
+    const uint64_t groups = (shots + 3) >> 2, stride = (uint64_t)gridDim.x * blockDim.x;
+    for (uint64_t g0 = (uint64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); g0 < groups; g0 += stride) {
+        const uint64_t g = g0 + lane;
+        const int cnt = g >= groups ? 0 : (int)min((uint64_t)4, shots - 4 * g);  // this lane's shots
+        double t[4];
+        uint32_t lo[4], hi[4];
+        if (u_in) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) t[k] = k < cnt ? u_in[4 * g + k] : 0.0;
+        } else {
+            uint64_t c[4] = {g, 0, 0, 0};
+            philox4x64_10(c, seed, 0);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) t[k] = (double)(c[k] >> 11) * 0x1.0p-53;
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const uint32_t i = (uint32_t)(t[k] * scale);  // u < 1: i < N
+            lo[k] = guide[i];
+            hi[k] = guide[i + 1];
+            t[k] *= S;
+        }
+        unsigned slow = 0;
+        uint64_t x[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            uint32_t a = lo[k], b = hi[k];
+            while (a < b) {
+                const uint32_t mid = (a + b) >> 1;
+                if (fine[mid] > t[k]) b = mid;
+                else a = mid + 1;
+            }
+            x[k] = a;
+            const double prev = a ? fine[a - 1] : -1.0;
+            // (a NaN total or table fails the compares and goes the slow way)
+            if (k < cnt && !(fine[a] > t[k] + d && (prev < t[k] - d || a == 0))) slow |= 1u << k;
+        }
+        for (unsigned m = __ballot_sync(0xffffffffu, slow != 0); m; m &= m - 1) {
+            const int src = __ffs(m) - 1;
+            const unsigned ks = __shfl_sync(0xffffffffu, slow, src);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                if (!((ks >> k) & 1)) continue;
+                const double ts = __shfl_sync(0xffffffffu, t[k], src);
+                const uint64_t j = warp_find_block(cdf, nblocks, ts, lane);
+                const uint64_t r = warp_sample<V>(amp, 5, cdf, j, S, ts, lane);
+                if (lane == src) x[k] = r;
+            }
+        }
+        if (cnt == 4) {
+            ulonglong2* o = (ulonglong2*)(out + 4 * g);
+            if (((uintptr_t)out & 15) == 0) {
+                o[0] = make_ulonglong2(x[0], x[1]);
+                o[1] = make_ulonglong2(x[2], x[3]);
                 continue;
             }
         }
-        double base = before;
-        for (uint64_t c = 0; c < len; c += 32) {
-            const bool valid = c + lane < len;
-            const double p = valid ? prob(amp(b0 + c + lane)) : 0.0;
-            double inc = p;
 #pragma unroll
-            for (int sh = 1; sh < 32; sh <<= 1) {
-                const double y = __shfl_up_sync(0xffffffffu, inc, sh);
-                if (lane >= sh) inc += y;
-            }
-            const unsigned hit = __ballot_sync(0xffffffffu, valid && p > 0.0 && base + inc > t);
-            if (hit) {
-                pick = b0 + c + (uint64_t)(__ffs(hit) - 1);
-                break;
-            }
-            const unsigned nz = __ballot_sync(0xffffffffu, p > 0.0);
-            if (nz) last_nz = b0 + c + (uint64_t)(31 - __clz(nz));  // fallback when rounding leaves no x above t
-            base += __shfl_sync(0xffffffffu, inc, 31);
-        }
-        if (lane == 0) out[s] = pick == UINT64_MAX ? last_nz : pick;
+        for (int k = 0; k < 4; ++k)
+            if (k < cnt) out[4 * g + k] = x[k];
     }
 }
 
@@ -581,17 +815,17 @@ int sample_blog(int n, uint64_t shots) {
 }
 }  // namespace
 
-// Inclusive FP64 scan of a[0..len) in place; chunks: (len + kScanCh - 1) / kScanCh doubles of scratch.
-static void scan_in_place(double* a, size_t len, double* chunks, cudaStream_t st) {
+// Inclusive FP64 scan of a[0..len) into out (may be a); chunks: (len + kScanCh - 1) / kScanCh doubles of scratch.
+static void scan_blocks(const double* a, double* out, size_t len, double* chunks, cudaStream_t st) {
     const size_t nch = (len + kScanCh - 1) / kScanCh;
     if (nch <= 1) {
         count_launch();
-        k_scan_chunks<<<1, kScanT, 0, st>>>(a, len, nullptr);
+        k_scan_chunks<<<1, kScanT, 0, st>>>(a, out, len, nullptr);
     } else {
         count_launch(3);
         k_chunk_totals<<<(unsigned)nch, kScanT, 0, st>>>(a, len, chunks);
         k_scan_totals<<<1, kScanT, 0, st>>>(chunks, (int)nch);
-        k_scan_chunks<<<(unsigned)nch, kScanT, 0, st>>>(a, len, chunks);
+        k_scan_chunks<<<(unsigned)nch, kScanT, 0, st>>>(a, out, len, chunks);
     }
 }
 
@@ -642,7 +876,7 @@ static int logical_block_cdf(sv_state* h, int blog, double** cdf_out, int64_t* n
         k_block_tot_logical<float2><<<g, 256, 0, h->stream>>>((const float2*)h->amps, lb, nunits, cdf);
     else
         k_block_tot_logical<double2><<<g, 256, 0, h->stream>>>((const double2*)h->amps, lb, nunits, cdf);
-    scan_in_place(cdf, nb, cdf + nb, h->stream);
+    scan_blocks(cdf, cdf, nb, cdf + nb, h->stream);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "logical block statistics");
     *cdf_out = cdf;
@@ -651,29 +885,31 @@ static int logical_block_cdf(sv_state* h, int blog, double** cdf_out, int64_t* n
 }
 
 // Block statistics in h->red: [raw block totals: nb][inclusive CDF: nb]
-// [chunk totals: nch][bit sums: 10 nb, when asked for].
+// [chunk totals: nch][bit sums: 10 nb, when asked for][quarter totals: 4 nb,
+// when asked for and the kernel has them; else *quart_out = nullptr].
 static int block_stats(sv_state* h, bool want_bits, double** tot_out, double** cdf_out, double** bits_out,
-                       int* blog_out, int64_t* nb_out, int blog_cap = kBlogMax) {
+                       int* blog_out, int64_t* nb_out, int blog_cap = kBlogMax, double** quart_out = nullptr) {
     int blog;
     const size_t nb = nblocks_of(h->n, &blog, blog_cap);
     const size_t nch = (nb + kScanCh - 1) / kScanCh;
-    const size_t need = sizeof(double) * (2 * nb + nch + 64 + (want_bits ? 10 * nb : 0));
+    const bool quarters = quart_out && want_bits && h->dtype == SV_C64 && blog == kBlogMax;
+    const size_t need = sizeof(double) * (2 * nb + nch + 64 + (want_bits ? 10 * nb : 0) + (quarters ? 4 * nb : 0));
     int rc = ensure_scratch(&h->red, need, h->stream);
     if (rc) return rc;
     double* tot = (double*)h->red.ptr;
     double* cdf = tot + nb;
     double* chunks = cdf + nb;
     double* bits = want_bits ? chunks + nch + 64 : nullptr;
+    double* quart = quarters ? bits + 10 * nb : nullptr;
+    if (quart_out) *quart_out = quart;
     const unsigned g = (unsigned)((nb * 32 + 255) / 256);
     count_launch();
     if (h->dtype == SV_C64)
-        k_block_stats<float2><<<g, 256, 0, h->stream>>>((const float2*)h->amps, blog, nb, tot, bits);
+        k_block_stats<float2><<<g, 256, 0, h->stream>>>((const float2*)h->amps, blog, nb, tot, bits, quart);
     else
-        k_block_stats<double2><<<g, 256, 0, h->stream>>>((const double2*)h->amps, blog, nb, tot, bits);
-    cudaError_t e = cudaMemcpyAsync(cdf, tot, sizeof(double) * nb, cudaMemcpyDeviceToDevice, h->stream);
-    if (e != cudaSuccess) return cuda_fail(e, "block totals copy");
-    scan_in_place(cdf, nb, chunks, h->stream);
-    e = cudaGetLastError();
+        k_block_stats<double2><<<g, 256, 0, h->stream>>>((const double2*)h->amps, blog, nb, tot, bits, nullptr);
+    scan_blocks(tot, cdf, nb, chunks, h->stream);
+    const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "block statistics");
     if (tot_out) *tot_out = tot;
     *cdf_out = cdf;
@@ -769,24 +1005,63 @@ int measure_norm(sv_state* h, double* host_out) {
     return SV_OK;
 }
 
+// The table pays once the shots number a quarter of the amplitudes: it reads
+// 8 bytes and writes 12 per amplitude (about 40 us at 2^20 amplitudes), a shot
+// without it takes about 1 ns.  Up to 2^24 amplitudes (200 MB).
+constexpr int kDenseMaxQubits = 24;
+static bool dense_shots(int n, int blog, uint64_t shots) {
+    return blog == 5 && n >= 10 && n <= kDenseMaxQubits && shots >= (1ull << n) / 4;
+}
+
+template <typename V, bool PERM>
+static void dense_t(sv_state* h, const double* cdf, int64_t nb, uint64_t shots, uint64_t seed, const double* dev_u,
+                    uint64_t* dev_out, const QubitMap& map) {
+    const V* a = (const V*)h->amps;
+    const uint32_t N = 1u << h->n;
+    double* fine = (double*)h->fine.ptr;
+    uint32_t* guide = (uint32_t*)(fine + N);
+    const unsigned cap = (unsigned)sms() * 8;
+    const unsigned gf = (unsigned)std::min<uint64_t>(((uint64_t)nb * 32 + 255) / 256, cap);
+    const unsigned gs = (unsigned)std::min<uint64_t>(((shots + 3) / 4 + 255) / 256, cap);
+    count_launch(3);
+    k_fine_cdf<V, PERM><<<gf, 256, 0, h->stream>>>(a, cdf, (uint64_t)nb, fine, map);
+    k_guide<<<gf, 256, 0, h->stream>>>(fine, N, guide);
+    k_sample_dense<V, PERM><<<gs, 256, 0, h->stream>>>(a, cdf, (uint64_t)nb, fine, guide, shots, seed, dev_u, dev_out,
+                                                      map);
+}
+
 // Shots from a block CDF; logical = the CDF is in logical order (relabelled
-// state) and the outcomes come out as logical indices.
+// state) and the outcomes come out as logical indices.  quart: see k_sample.
 static cudaError_t launch_sample(sv_state* h, int blog, const double* cdf, int64_t nb, uint64_t shots,
-                                 uint64_t seed, const double* dev_u, uint64_t* dev_out, bool logical = false) {
+                                 uint64_t seed, const double* dev_u, uint64_t* dev_out, bool logical = false,
+                                 const double* quart = nullptr) {
+    const QubitMap map = qubit_map(h);
+    // (without memory for the table the shots go one warp at a time)
+    if (dense_shots(h->n, blog, shots) &&
+        ensure_scratch(&h->fine, (sizeof(double) << h->n) + sizeof(uint32_t) * ((1ull << h->n) + 1), h->stream) == SV_OK) {
+        if (h->dtype == SV_C64) {
+            if (logical) dense_t<float2, true>(h, cdf, nb, shots, seed, dev_u, dev_out, map);
+            else dense_t<float2, false>(h, cdf, nb, shots, seed, dev_u, dev_out, map);
+        } else {
+            if (logical) dense_t<double2, true>(h, cdf, nb, shots, seed, dev_u, dev_out, map);
+            else dense_t<double2, false>(h, cdf, nb, shots, seed, dev_u, dev_out, map);
+        }
+        return cudaGetLastError();
+    }
     uint64_t g = (shots * 32 + 255) / 256;
     const uint64_t cap = (uint64_t)sms() * 16;
     if (g > cap) g = cap;
     count_launch();
-    const QubitMap map = qubit_map(h);
     const unsigned gg = (unsigned)g;
+    const uint64_t n = (uint64_t)nb;
     if (h->dtype == SV_C64) {
         const float2* a = (const float2*)h->amps;
-        if (logical) k_sample<float2, true><<<gg, 256, 0, h->stream>>>(a, h->n, blog, cdf, nb, shots, seed, dev_u, dev_out, map);
-        else k_sample<float2, false><<<gg, 256, 0, h->stream>>>(a, h->n, blog, cdf, nb, shots, seed, dev_u, dev_out, map);
+        if (logical) k_sample<float2, true><<<gg, 256, 0, h->stream>>>(a, blog, cdf, n, nullptr, shots, seed, dev_u, dev_out, map);
+        else k_sample<float2, false><<<gg, 256, 0, h->stream>>>(a, blog, cdf, n, quart, shots, seed, dev_u, dev_out, map);
     } else {
         const double2* a = (const double2*)h->amps;
-        if (logical) k_sample<double2, true><<<gg, 256, 0, h->stream>>>(a, h->n, blog, cdf, nb, shots, seed, dev_u, dev_out, map);
-        else k_sample<double2, false><<<gg, 256, 0, h->stream>>>(a, h->n, blog, cdf, nb, shots, seed, dev_u, dev_out, map);
+        if (logical) k_sample<double2, true><<<gg, 256, 0, h->stream>>>(a, blog, cdf, n, nullptr, shots, seed, dev_u, dev_out, map);
+        else k_sample<double2, false><<<gg, 256, 0, h->stream>>>(a, blog, cdf, n, nullptr, shots, seed, dev_u, dev_out, map);
     }
     return cudaGetLastError();
 }
@@ -805,10 +1080,11 @@ static int sample_logical(sv_state* h, int blog, uint64_t shots, uint64_t seed, 
 
 // Shots and <Z_i> from ONE pass over the state (either output may be NULL).
 int measure_readout(sv_state* h, uint64_t shots, uint64_t seed, uint64_t* dev_samples, double* dev_expz) {
-    double *tot, *cdf, *bits;
+    double *tot, *cdf, *bits, *quart = nullptr;
     int blog;
     int64_t nb;
-    int rc = block_stats(h, dev_expz != nullptr, &tot, &cdf, &bits, &blog, &nb);
+    const bool here = dev_samples && shots && !h->permuted;  // shots drawn from these blocks
+    int rc = block_stats(h, dev_expz != nullptr, &tot, &cdf, &bits, &blog, &nb, kBlogMax, here ? &quart : nullptr);
     if (rc) return rc;
     if (dev_expz) {
         // chunk partials, then (relabelled qubits) the physical-bit values
@@ -830,7 +1106,7 @@ int measure_readout(sv_state* h, uint64_t shots, uint64_t seed, uint64_t* dev_sa
         // a relabelled state samples from its logical-order CDF (a second
         // read of the state; <Z> above used the physical block statistics)
         if (h->permuted) return sample_logical(h, blog, shots, seed, nullptr, dev_samples);
-        e = launch_sample(h, blog, cdf, nb, shots, seed, nullptr, dev_samples);
+        e = launch_sample(h, blog, cdf, nb, shots, seed, nullptr, dev_samples, false, quart);
         if (e != cudaSuccess) return cuda_fail(e, "read-out");
     }
     return SV_OK;
@@ -926,28 +1202,28 @@ extern "C" int sv_sample_uniforms_noalloc(const void* dev_amps, int n, sv_dtype 
     const unsigned g = (unsigned)((nb * 32 + 255) / 256);
     count_launch();
     if (dt == SV_C64)
-        k_block_stats<float2><<<g, 256, 0, st>>>((const float2*)dev_amps, blog, nb, bs, nullptr);
+        k_block_stats<float2><<<g, 256, 0, st>>>((const float2*)dev_amps, blog, nb, bs, nullptr, nullptr);
     else
-        k_block_stats<double2><<<g, 256, 0, st>>>((const double2*)dev_amps, blog, nb, bs, nullptr);
+        k_block_stats<double2><<<g, 256, 0, st>>>((const double2*)dev_amps, blog, nb, bs, nullptr, nullptr);
     if (nch <= 1) {
         count_launch();
-        k_scan_chunks<<<1, kScanT, 0, st>>>(bs, nb, nullptr);
+        k_scan_chunks<<<1, kScanT, 0, st>>>(bs, bs, nb, nullptr);
     } else {
         count_launch(3);
         k_chunk_totals<<<(unsigned)nch, kScanT, 0, st>>>(bs, nb, tot);
         k_scan_totals<<<1, kScanT, 0, st>>>(tot, (int)nch);
-        k_scan_chunks<<<(unsigned)nch, kScanT, 0, st>>>(bs, nb, tot);
+        k_scan_chunks<<<(unsigned)nch, kScanT, 0, st>>>(bs, bs, nb, tot);
     }
     uint64_t gs = (shots * 32 + 255) / 256;
     const uint64_t cap = (uint64_t)sms() * 16;
     if (gs > cap) gs = cap;
     count_launch();
     if (dt == SV_C64)
-        k_sample<float2, false><<<(unsigned)gs, 256, 0, st>>>((const float2*)dev_amps, n, blog, bs, (uint64_t)nb,
+        k_sample<float2, false><<<(unsigned)gs, 256, 0, st>>>((const float2*)dev_amps, blog, bs, (uint64_t)nb, nullptr,
                                                              shots, 0, dev_u, dev_out, QubitMap{});
     else
-        k_sample<double2, false><<<(unsigned)gs, 256, 0, st>>>((const double2*)dev_amps, n, blog, bs,
-                                                              (uint64_t)nb, shots, 0, dev_u, dev_out, QubitMap{});
+        k_sample<double2, false><<<(unsigned)gs, 256, 0, st>>>((const double2*)dev_amps, blog, bs, (uint64_t)nb,
+                                                              nullptr, shots, 0, dev_u, dev_out, QubitMap{});
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "sv_sample_uniforms_noalloc");
     return SV_OK;
