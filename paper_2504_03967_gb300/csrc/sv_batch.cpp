@@ -470,20 +470,24 @@ extern "C" int sv_batch_run(int C, const int* n_qubits, const int64_t* gate_offs
             }
             void* base = nullptr;
             rc = enqueue_wave(dt, w, st, kWaveWaitLimit, d_err, &keep, &base);
-            if (rc == SV_OK) {  // the read-out streams start after the wave
+            if (rc == SV_OK && host_expz) {  // all circuits of the wave at once
+                std::vector<double*> rows;
+                for (int c : wc) rows.push_back(d_expz + (size_t)slot[c] * nmax);
+                rc = measure_expz_many(dt, base, (int)wc.size(), w.offs.data(), w.nq.data(), w.amps, rows.data(), st,
+                                       &keep.pinned);
+            }
+            if (rc == SV_OK && host_samples) {  // the sampling streams start after the wave
                 cudaEventRecord(vev, st);
                 for (int v = 0; v < kViews; ++v) cudaStreamWaitEvent(vs[v], vev, 0);
             }
-            for (size_t k = 0; rc == SV_OK && k < wc.size(); ++k) {
+            for (size_t k = 0; rc == SV_OK && host_samples && k < wc.size(); ++k) {
                 const int c = wc[k];
                 const int idx = slot[c];
                 sv_state& h = hv[k % kViews];
                 h.n = n_qubits[c];
                 h.amps = (char*)base + csz * w.offs[k];
                 reset_perm(&h);
-                if (host_samples)
-                    rc = measure_sample(&h, shots, seed + (uint64_t)c, nullptr, d_samples + (size_t)idx * shots);
-                if (rc == SV_OK && host_expz) rc = measure_expect_z(&h, d_expz + (size_t)idx * nmax);
+                rc = measure_sample(&h, shots, seed + (uint64_t)c, nullptr, d_samples + (size_t)idx * shots);
             }
             for (int v = 0; v < kViews; ++v) {  // the wave's buffer is freed after its read-outs
                 cudaEventRecord(vev, vs[v]);

@@ -456,6 +456,11 @@ cudaError_t launch_probs(sv_state* h, double* dev_out);
 cudaError_t launch_gather_logical(sv_state* h, uint64_t x0, uint64_t cnt, void* dev_out);
 int measure_norm(sv_state* h, double* host_out);
 int measure_expect_z(sv_state* h, double* dev_out);
+// <Z_i> of a wave's states (offs[c] amplitudes from base, n[c] >= 10 qubits,
+// amps amplitudes in all) into rows[c], three launches on st; pinned: staging
+// to free once st has been synchronised.
+int measure_expz_many(int dtype, const void* base, int C, const uint64_t* offs, const int* n, uint64_t amps,
+                      double* const* rows, cudaStream_t st, std::vector<void*>* pinned);
 // Shots and <Z_i> from one pass over the state (either output may be NULL).
 int measure_readout(sv_state* h, uint64_t shots, uint64_t seed, uint64_t* dev_samples, double* dev_expz);
 

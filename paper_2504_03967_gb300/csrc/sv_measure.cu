@@ -10,6 +10,9 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <string.h>
+
+#include <algorithm>
 #include <mutex>
 #include <string>
 
@@ -40,7 +43,8 @@ __device__ __forceinline__ double warp_sum(double v) {
 // block value carries the same information as an FP64 sum, at FP32 speed
 // (this GPU's FP64 rate is a small fraction of its FP32 rate).  complex128
 // accumulates in FP64.  bits (optional, nblocks x 10) receives, for each
-// block, the probability mass with index bit i set, i < min(blog, 10).
+// block (complex64, blog = 10: for each CTA's 8 blocks together), the
+// probability mass with index bit i set, i < min(blog, 10).
 struct FF {
     float hi, lo;
 };
@@ -84,8 +88,8 @@ __device__ __forceinline__ FF ff_allreduce(FF a) {
 // first four exchange steps halves the values a lane keeps, so lane 2e
 // (e < 14) ends with value e summed over all 32 lanes.
 __device__ __forceinline__ void block_stats_c64_full(const float2* __restrict__ psi, uint64_t wid, int lane,
-                                                     double* __restrict__ tot, double* __restrict__ bits,
-                                                     double* __restrict__ quart) {
+                                                     double* __restrict__ tot, FF* __restrict__ sbits,
+                                                     float2* __restrict__ quart) {
     const uint64_t b0 = wid << 10;
     FF p[32];
 #pragma unroll
@@ -136,19 +140,20 @@ __device__ __forceinline__ void block_stats_c64_full(const float2* __restrict__ 
         }
     }
     ff_add(e[0], __shfl_xor_sync(0xffffffffu, e[0].hi, 1), __shfl_xor_sync(0xffffffffu, e[0].lo, 1));
+    // value idx: 0 total; 1..5 lane bits 0..4; 6..10 j bits = index bits 5..9; 11..13 quarters
     const int idx = ((lane >> 4) & 1) * 8 + ((lane >> 3) & 1) * 4 + ((lane >> 2) & 1) * 2 + ((lane >> 1) & 1);
-    if (!(lane & 1) && idx < 14) {
-        const double val = ff_val(e[0]);
-        if (idx == 0) tot[wid] = val;
-        else if (idx < 11) bits[wid * 10 + (idx - 1)] = val;  // 1..5: lane bits 0..4; 6..10: j bits = index bits 5..9
-        else if (quart) quart[wid * 4 + (idx - 11)] = val;
+    if (lane == 0) tot[wid] = ff_val(e[0]);
+    if (!(lane & 1)) {
+        if (idx >= 11 && idx < 14 && quart) quart[wid * 4 + (idx - 11)] = make_float2(e[0].hi, e[0].lo);
+        if (idx >= 1 && idx < 11) sbits[(threadIdx.x >> 5) * 10 + idx - 1] = e[0];
     }
 }
+constexpr int kBitsGroupLog = 3;  // complex64 bit sums: one record per CTA of k_block_stats (8 blocks)
 
 template <typename V>
 __global__ void __launch_bounds__(256) k_block_stats(const V* __restrict__ psi, int blog, uint64_t nblocks,
                                                      double* __restrict__ tot, double* __restrict__ bits,
-                                                     double* __restrict__ quart) {
+                                                     float2* __restrict__ quart) {
     const int lane = threadIdx.x & 31;
     const uint64_t wid = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (wid >= nblocks) return;
@@ -157,7 +162,19 @@ __global__ void __launch_bounds__(256) k_block_stats(const V* __restrict__ psi, 
     const int jn = len >= 32 ? len / 32 : 1;
     if constexpr (sizeof(V) == 8) {
         if (bits && blog == 10) {
-            block_stats_c64_full((const float2*)psi, wid, lane, tot, bits, quart);
+            __shared__ FF sbits[80];
+            block_stats_c64_full((const float2*)psi, wid, lane, tot, sbits, quart);
+            if (nblocks < 8) {  // (one partly filled CTA: a record per block)
+                __syncwarp();
+                if (lane < 10) bits[wid * 10 + lane] = ff_val(sbits[(threadIdx.x >> 5) * 10 + lane]);
+                return;
+            }
+            __syncthreads();  // (nblocks is a multiple of 8: every warp is here)
+            if (threadIdx.x < 10) {
+                FF v = sbits[threadIdx.x];
+                for (int w = 1; w < 8; ++w) ff_add(v, sbits[10 * w + threadIdx.x].hi, sbits[10 * w + threadIdx.x].lo);
+                bits[(uint64_t)blockIdx.x * 10 + threadIdx.x] = ff_val(v);
+            }
             return;
         }
         FF acc = {0.f, 0.f}, ab[5];
@@ -219,47 +236,115 @@ __global__ void __launch_bounds__(256) k_block_stats(const V* __restrict__ psi, 
     }
 }
 
-// <Z_i> = S - 2 * (mass with bit i set) from the block records.  Stage 1:
-// CTA (i, g) reduces chunk g of the block records for qubit i (fixed order);
-// stage 2: one thread per qubit adds its chunk partials in order.
-constexpr int kExpzChunks = 64;
-__global__ void __launch_bounds__(256) k_expz_blocks(const double* __restrict__ tot, const double* __restrict__ bits,
-                                                     uint64_t nblocks, int blog, double* __restrict__ part) {
-    __shared__ double s1[256], s2[256];
-    const int i = blockIdx.x, g = blockIdx.y;
-    const uint64_t per = (nblocks + kExpzChunks - 1) / kExpzChunks;
-    const uint64_t k0 = (uint64_t)g * per, k1 = k0 + per < nblocks ? k0 + per : nblocks;
-    double a = 0.0, b = 0.0;
-    for (uint64_t k = k0 + threadIdx.x; k < k1; k += blockDim.x) {
-        const double tk = tot[k];
-        a += tk;
-        if (i < blog) b += bits[k * 10 + i];
-        else if ((k >> (i - blog)) & 1) b += tk;
+// <Z_i> = S - 2 * (mass with bit i set) from the block records of one or
+// several states (item = blockIdx.y).  Stage 1: CTA g reduces 2^lper
+// consecutive block records once, for all qubits: the total, the bit sums
+// below blog (read flat, ten doubles per record of 2^bg blocks, thread t
+// always at the same bit), and the totals of the records whose index has bit
+// b set, b < lper.  Stage 2: one warp per qubit adds the CTAs' partials (a
+// record-index bit at or above lper selects whole CTAs).  All sums have a
+// fixed order.  Bound by the FP64 pipe (one warp add per 78 clocks and
+// scheduler on this GPU), so the warp sums go through one reduce-scatter (16
+// adds for 16 values) and the bit sums arrive added over 8 blocks in
+// double-float; one CTA per qubit and chunk reading every block's ten sums
+// took 63 us at 2^18 records.
+struct ExpzItem {
+    uint64_t blk0;    // first block record of the state
+    uint64_t nb;      // its records (a power of two)
+    int n, blog;      // qubits; amplitudes per record 2^blog
+    int lper, lg;     // records per CTA 2^lper, CTAs 2^lg (nb = 2^(lper + lg))
+    int bg;           // bit sums cover 2^bg records
+    uint64_t out;     // offset of its n values in the output
+};
+constexpr int kExpzMaxLg = 8;     // at most 256 CTAs per state
+constexpr int kExpzSlots = 32;    // partials of one CTA: total | bit sums [10] | index-bit sums [lper <= 16]
+
+// all: blocks of the k_block_stats launch the records come from
+ExpzItem expz_item(uint64_t blk0, uint64_t nb, int n, int blog, uint64_t out, int dtype, uint64_t all) {
+    ExpzItem I{blk0, nb, n, blog, 0, 0, 0, out};
+    int l = 0;
+    while ((1ull << l) < nb) ++l;
+    I.lg = std::max(0, std::min(kExpzMaxLg, l - 8));  // at least 256 records per CTA
+    I.lper = l - I.lg;
+    I.bg = dtype == SV_C64 && blog == kBlogMax && all >= 8 ? kBitsGroupLog : 0;
+    return I;
+}
+
+__global__ void __launch_bounds__(256) k_expz_part(const double* __restrict__ tot, const double* __restrict__ bits,
+                                                   const ExpzItem* __restrict__ items, const ExpzItem one,
+                                                   double* __restrict__ part) {
+    __shared__ double sb[256], sw[8][16];
+    const ExpzItem I = items ? items[blockIdx.y] : one;
+    if (blockIdx.x >> I.lg) return;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint64_t per = 1ull << I.lper, k0 = I.blk0 + ((uint64_t)blockIdx.x << I.lper);
+    double* out = part + ((uint64_t)blockIdx.y * gridDim.x + blockIdx.x) * kExpzSlots;
+    double bsum = 0.0;
+    if (tid < 250) {
+        const double* src = bits + (k0 >> I.bg) * 10;
+        const uint64_t cnt = (per >> I.bg) * 10;
+#pragma unroll 4
+        for (uint64_t e = tid; e < cnt; e += 250) bsum += src[e];
     }
-    s1[threadIdx.x] = a;
-    s2[threadIdx.x] = b;
-    __syncthreads();
-    for (int w = 128; w > 0; w >>= 1) {
-        if ((int)threadIdx.x < w) {
-            s1[threadIdx.x] += s1[threadIdx.x + w];
-            s2[threadIdx.x] += s2[threadIdx.x + w];
+    sb[tid] = bsum;
+    // record k = tid + 256 r: its index bits 0..4 are the lane, 5..7 the warp,
+    // the others r.  e: total | lane bits | r bits (at most 8: lper <= 16)
+    double e[16];
+#pragma unroll
+    for (int b = 0; b < 16; ++b) e[b] = 0.0;
+    for (uint64_t r = 0; tid + 256 * r < per; ++r) {
+        const double v = tot[k0 + tid + 256 * r];
+        e[0] += v;
+#pragma unroll
+        for (int b = 0; b < 8; ++b)
+            if ((r >> b) & 1) e[6 + b] += v;
+    }
+#pragma unroll
+    for (int b = 0; b < 5; ++b) e[1 + b] = ((lane >> b) & 1) ? e[0] : 0.0;
+#pragma unroll
+    for (int st = 0; st < 4; ++st) {  // lane bits 4, 3, 2, 1: each step halves the values a lane keeps
+        const int hv = 8 >> st, mask = 16 >> st;
+        const bool up = (lane & mask) != 0;
+#pragma unroll
+        for (int k = 0; k < hv; ++k) {
+            const double send = up ? e[k] : e[k + hv], keep = up ? e[k + hv] : e[k];
+            e[k] = keep + __shfl_xor_sync(0xffffffffu, send, mask);
         }
-        __syncthreads();
     }
-    if (threadIdx.x == 0) {
-        part[2 * (i * kExpzChunks + g)] = s1[0];
-        part[2 * (i * kExpzChunks + g) + 1] = s2[0];
+    e[0] += __shfl_xor_sync(0xffffffffu, e[0], 1);
+    if (!(lane & 1)) sw[warp][((lane >> 4) & 1) * 8 + ((lane >> 3) & 1) * 4 + ((lane >> 2) & 1) * 2 + ((lane >> 1) & 1)] = e[0];
+    __syncthreads();
+    // slot tid of the partials; index bits 0..4 are values 1..5, 5..7 the warps, 8.. values 6..
+    if (tid == 0 || (tid >= 11 && tid < 11 + I.lper)) {
+        const int b = tid - 11;
+        double v = 0.0;
+        for (int w = 0; w < 8; ++w)
+            if (tid == 0 || b < 5 || b >= 8) v += sw[w][tid == 0 ? 0 : b < 5 ? 1 + b : b - 2];
+            else if ((w >> (b - 5)) & 1) v += sw[w][0];
+        out[tid] = v;
+    } else if (tid >= 32 && tid < 42) {
+        double v = 0.0;
+        for (int i = tid - 32; i < 250; i += 10) v += sb[i];
+        out[tid - 31] = v;
     }
 }
-__global__ void k_expz_final(const double* __restrict__ part, int n, double* __restrict__ out) {
-    const int i = threadIdx.x;
-    if (i >= n) return;
+__global__ void __launch_bounds__(32) k_expz_sum(const double* __restrict__ part, const ExpzItem* __restrict__ items,
+                                                 const ExpzItem one, int gmax, double* __restrict__ out) {
+    const ExpzItem I = items ? items[blockIdx.y] : one;
+    const int i = blockIdx.x, lane = threadIdx.x;
+    if (i >= I.n) return;
+    const double* src = part + (uint64_t)blockIdx.y * gmax * kExpzSlots;
+    const int kb = i - I.blog;  // record-index bit of qubit i (below 0: a bit sum)
     double a = 0.0, b = 0.0;
-    for (int g = 0; g < kExpzChunks; ++g) {
-        a += part[2 * (i * kExpzChunks + g)];
-        b += part[2 * (i * kExpzChunks + g) + 1];
+    for (int g = lane; g < (1 << I.lg); g += 32) {
+        const double* p = src + g * kExpzSlots;
+        a += p[0];
+        if (kb < 0) b += p[1 + i];
+        else if (kb < I.lper) b += p[11 + kb];
+        else if ((g >> (kb - I.lper)) & 1) b += p[0];
     }
-    out[i] = a - 2.0 * b;
+    const double v = warp_sum(a - 2.0 * b);
+    if (lane == 0) out[I.out + i] = v;
 }
 
 // ---- inclusive scan of doubles -------------------------------------------
@@ -467,9 +552,9 @@ __global__ void __launch_bounds__(256) k_block_tot_logical(const V* __restrict__
 //  * warp_sample: one warp per shot, the rule itself.  A 32-way search of the
 //    block CDF, then a rescan of the chosen block 32 amplitudes at a time (a
 //    coalesced load, a warp scan on top of the running CDF, a ballot).
-//  * warp_sample_quarter (complex64, 1024-amplitude blocks with quarter
-//    totals): the quarter totals leave 256 of the 1024 amplitudes to read,
-//    and one warp scan finds x among them.
+//  * k_sample_quarter (complex64, 1024-amplitude blocks with quarter totals):
+//    the quarter totals leave 256 of the 1024 amplitudes to read, and one warp
+//    scan finds x among them.
 //  * k_sample_dense (about as many shots as amplitudes, or more): a table of
 //    C_x for every x and a guide into it, one thread per shot.
 //
@@ -564,81 +649,14 @@ __device__ __forceinline__ uint64_t warp_sample(const Amp& amp, int blog, const 
     return pick == UINT64_MAX ? last_nz : pick;
 }
 
-// Block j (1024 amplitudes of complex64) with its quarter totals: the quarter
-// from its totals, then lane l adds the quarter's amplitudes 8 l .. 8 l + 7 (64
-// contiguous bytes, 2 KB per warp), one warp scan of the lane sums picks the
-// lane, and its eight probabilities, sent to all lanes, give x.  All compares
-// are against t minus the quarter's start, in double-float (a float pair holds
-// 48 bits of a value of at most S, far below kClear S).  UINT64_MAX: t is not
-// clear of the neighbouring outcomes.  Bound by the 2 KB read per shot; with
-// the whole block (8 KB, 32 dependent scan steps of which half are taken on
-// average) 10^5 shots of a 28-qubit state took 339 us.
-__device__ __forceinline__ uint64_t warp_sample_quarter(const float2* __restrict__ psi, const double* __restrict__ cdf,
-                                                        const double* __restrict__ quart, uint64_t j, double S, double t,
-                                                        int lane) {
-    const double before = j ? cdf[j - 1] : 0.0;
-    double r = t - before;  // what is left of t inside the block
-    int q = 0;
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {  // (uniform across the warp)
-        const double w = quart[j * 4 + k];
-        if (q == k && r >= w) {
-            r -= w;
-            q = k + 1;
-        }
-    }
-    const float4* src = (const float4*)(psi + (j << 10) + (q << 8)) + 4 * lane;
-    FF p[8], sum{0.f, 0.f};
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const float4 v = src[i];
-        p[2 * i] = ff_prob(make_float2(v.x, v.y));
-        p[2 * i + 1] = ff_prob(make_float2(v.z, v.w));
-    }
-#pragma unroll
-    for (int i = 0; i < 8; ++i) ff_add(sum, p[i].hi, p[i].lo);
-    FF inc = sum;
-#pragma unroll
-    for (int sh = 1; sh < 32; sh <<= 1) {
-        const float h = __shfl_up_sync(0xffffffffu, inc.hi, sh);
-        const float l = __shfl_up_sync(0xffffffffu, inc.lo, sh);
-        if (lane >= sh) ff_add(inc, h, l);
-    }
-    const FF rf = ff_of(r);
-    const unsigned over = __ballot_sync(0xffffffffu, (inc.hi - rf.hi) + (inc.lo - rf.lo) > 0.f);
-    if (!over) return UINT64_MAX;
-    const int f = __ffs(over) - 1;
-    FF cum{0.f, 0.f};
-    if (f) {
-        cum.hi = __shfl_sync(0xffffffffu, inc.hi, f - 1);
-        cum.lo = __shfl_sync(0xffffffffu, inc.lo, f - 1);
-    }
-    const float d = (float)(kClear * S);
-    float prev = (cum.hi - rf.hi) + (cum.lo - rf.lo);  // C_{x-1} - t
-    int at = 8;
-    bool clear = false;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        ff_add(cum, __shfl_sync(0xffffffffu, p[i].hi, f), __shfl_sync(0xffffffffu, p[i].lo, f));
-        const float cur = (cum.hi - rf.hi) + (cum.lo - rf.lo);
-        if (at == 8 && cur > 0.f) {
-            at = i;
-            clear = prev < -d && cur > d;
-        }
-        prev = cur;
-    }
-    return clear ? (j << 10) + (uint64_t)(q << 8) + 8 * f + at : UINT64_MAX;
-}
-
 // PERM (a relabelled state): cdf is the block CDF in LOGICAL order (from
 // k_block_tot_logical) and the chosen block is rescanned in logical order,
 // amplitude x read at its physical index; the outcome is the logical x.
-// quart: quarter totals of the blocks (complex64, blog = 10), or nullptr.
 template <typename V, bool PERM>
 __global__ void __launch_bounds__(256) k_sample(const V* __restrict__ psi, int blog, const double* __restrict__ cdf,
-                                                uint64_t nblocks, const double* __restrict__ quart, uint64_t shots,
-                                                uint64_t seed, const double* __restrict__ u_in,
-                                                uint64_t* __restrict__ out, const QubitMap map) {
+                                                uint64_t nblocks, uint64_t shots, uint64_t seed,
+                                                const double* __restrict__ u_in, uint64_t* __restrict__ out,
+                                                const QubitMap map) {
     __shared__ uint64_t qt[PERM ? 5 : 1][256];
     if constexpr (PERM) {
         build_byte_tables(qt, map);
@@ -651,25 +669,128 @@ __global__ void __launch_bounds__(256) k_sample(const V* __restrict__ psi, int b
     const int lane = threadIdx.x & 31;
     const uint64_t warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
     const double S = cdf[nblocks - 1];
-    const bool short_cut = quart && S > 1e-20 && S < 1e20;
     for (uint64_t s = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; s < shots; s += warps) {
         const double u = u_in ? u_in[s] : philox_uniform(seed, s);
         const double t = u * S;
         const uint64_t j = warp_find_block(cdf, nblocks, t, lane);
-        uint64_t x = UINT64_MAX;
-        if constexpr (sizeof(V) == 8 && !PERM)
-            if (short_cut) x = warp_sample_quarter((const float2*)psi, cdf, quart, j, S, t, lane);
-        if (x == UINT64_MAX) x = warp_sample<V>(amp, blog, cdf, j, S, t, lane);
+        const uint64_t x = warp_sample<V>(amp, blog, cdf, j, S, t, lane);
         if (lane == 0) out[s] = x;
     }
 }
 
+// ---- few shots on a large complex64 state: quarter totals -----------------------
+// A warp takes G <= 32 shots at a time.  Lane k finds shot k's block by binary
+// search, its quarter from the quarter totals, and what is left of t there;
+// then the warp serves the shots one by one: lane l adds the quarter's
+// amplitudes 8 l .. 8 l + 7 (64 contiguous bytes, 2 KB per warp), one warp scan
+// of the lane sums picks the lane, and its eight probabilities, sent to all
+// lanes, give x.  All compares are against t minus the quarter's start, in
+// double-float (a float pair holds 48 bits of a value of at most S, far below
+// kClear S).  Everything in FP64 is done once per shot in one lane, because a
+// warp-wide FP64 instruction costs 78 clocks here (done by all lanes, these
+// were 120 of 140 us); block CDF entries are compared as integers (finite
+// doubles >= 0 order as their bits).  10^5 shots of a 28-qubit state with the
+// whole block rescanned by a warp per shot: 339 us.
+__global__ void __launch_bounds__(256) k_sample_quarter(const float2* __restrict__ psi, const double* __restrict__ cdf,
+                                                        uint64_t nblocks, const float2* __restrict__ quart, int G,
+                                                        uint64_t shots, uint64_t seed, uint64_t* __restrict__ out) {
+    const int lane = threadIdx.x & 31;
+    const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const uint64_t warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
+    const double S = cdf[nblocks - 1];
+    const bool sane = S > 1e-20 && S < 1e20;
+    const float d = (float)(kClear * S);
+    auto amp = [&](uint64_t x) { return psi[x]; };
+    for (uint64_t s0 = warp * G; s0 < shots; s0 += warps * G) {
+        const bool mine = lane < G && s0 + lane < shots;
+        double t = 0.0;
+        uint64_t j = 0, x = UINT64_MAX;
+        int q = 0;
+        FF rf{0.f, 0.f};
+        if (mine && sane) {
+            t = philox_uniform(seed, s0 + lane) * S;
+            const long long tb = __double_as_longlong(t);
+            uint64_t lo = 0, hi = nblocks - 1;
+            while (lo < hi) {
+                const uint64_t mid = (lo + hi) >> 1;
+                if (__double_as_longlong(cdf[mid]) > tb) hi = mid;
+                else lo = mid + 1;
+            }
+            j = lo;
+            rf = ff_of(t - (j ? cdf[j - 1] : 0.0));
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const float2 w = quart[j * 4 + k];
+                if (q == k && (rf.hi - w.x) + (rf.lo - w.y) >= 0.f) {
+                    ff_add(rf, -w.x, -w.y);
+                    q = k + 1;
+                }
+            }
+        } else if (mine) {
+            t = philox_uniform(seed, s0 + lane) * S;
+        }
+        const int cnt = (int)min((uint64_t)G, shots - s0);
+        if (sane) {
+            for (int k = 0; k < cnt; ++k) {
+                const uint64_t jk = __shfl_sync(0xffffffffu, j, k);
+                const int qk = __shfl_sync(0xffffffffu, q, k);
+                const FF rk{__shfl_sync(0xffffffffu, rf.hi, k), __shfl_sync(0xffffffffu, rf.lo, k)};
+                const float4* src = (const float4*)(psi + (jk << 10) + (qk << 8)) + 4 * lane;
+                FF p[8], sum{0.f, 0.f};
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float4 v = src[i];
+                    p[2 * i] = ff_prob(make_float2(v.x, v.y));
+                    p[2 * i + 1] = ff_prob(make_float2(v.z, v.w));
+                }
+#pragma unroll
+                for (int i = 0; i < 8; ++i) ff_add(sum, p[i].hi, p[i].lo);
+                FF inc = sum;
+#pragma unroll
+                for (int sh = 1; sh < 32; sh <<= 1) {
+                    const float h = __shfl_up_sync(0xffffffffu, inc.hi, sh);
+                    const float l = __shfl_up_sync(0xffffffffu, inc.lo, sh);
+                    if (lane >= sh) ff_add(inc, h, l);
+                }
+                const unsigned over = __ballot_sync(0xffffffffu, (inc.hi - rk.hi) + (inc.lo - rk.lo) > 0.f);
+                if (!over) continue;  // (uniform; the shot stays unanswered)
+                const int f = __ffs(over) - 1;
+                FF cum{__shfl_sync(0xffffffffu, inc.hi, f > 0 ? f - 1 : 0), __shfl_sync(0xffffffffu, inc.lo, f > 0 ? f - 1 : 0)};
+                if (f == 0) cum = FF{0.f, 0.f};
+                float prev = (cum.hi - rk.hi) + (cum.lo - rk.lo);  // C_{x-1} - t
+                int at = 8;
+                bool clear = false;
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    ff_add(cum, __shfl_sync(0xffffffffu, p[i].hi, f), __shfl_sync(0xffffffffu, p[i].lo, f));
+                    const float cur = (cum.hi - rk.hi) + (cum.lo - rk.lo);
+                    if (at == 8 && cur > 0.f) {
+                        at = i;
+                        clear = prev < -d && cur > d;
+                    }
+                    prev = cur;
+                }
+                if (lane == k && clear) x = (jk << 10) + (uint64_t)(qk << 8) + 8 * f + at;
+            }
+        }
+        for (unsigned m = __ballot_sync(0xffffffffu, mine && x == UINT64_MAX); m; m &= m - 1) {
+            const int k = __ffs(m) - 1;
+            const double tk = __shfl_sync(0xffffffffu, t, k);
+            const uint64_t r = warp_sample<float2>(amp, kBlogMax, cdf, warp_find_block(cdf, nblocks, tk, lane), S, tk, lane);
+            if (lane == k) x = r;
+        }
+        if (mine) out[s0 + lane] = x;
+    }
+}
+
 // ---- many shots: a table of the CDF ------------------------------------------
-// fine[x] = C_x for every amplitude (one warp per 32-amplitude block of the
-// block CDF, FP64) ...
+// fine[x] = C_x / S in units of 2^-53 for every amplitude (one warp per
+// 32-amplitude block of the block CDF; FP64, then rounded down to an integer,
+// which is what a uniform is: w 2^-53) ...
+constexpr double kTwo53 = 9007199254740992.0;
 template <typename V, bool PERM>
 __global__ void __launch_bounds__(256) k_fine_cdf(const V* __restrict__ psi, const double* __restrict__ cdf,
-                                                  uint64_t nblocks, double* __restrict__ fine, const QubitMap map) {
+                                                  uint64_t nblocks, uint64_t* __restrict__ fine, const QubitMap map) {
     __shared__ uint64_t qt[PERM ? 5 : 1][256];
     if constexpr (PERM) {
         build_byte_tables(qt, map);
@@ -677,6 +798,7 @@ __global__ void __launch_bounds__(256) k_fine_cdf(const V* __restrict__ psi, con
     }
     const int lane = threadIdx.x & 31;
     const uint64_t warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
+    const double S = cdf[nblocks - 1], scale = S > 0.0 ? kTwo53 / S : 0.0;
     for (uint64_t j = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; j < nblocks; j += warps) {
         const uint64_t x = (j << 5) + lane;
         double inc;
@@ -687,16 +809,17 @@ __global__ void __launch_bounds__(256) k_fine_cdf(const V* __restrict__ psi, con
             const double y = __shfl_up_sync(0xffffffffu, inc, sh);
             if (lane >= sh) inc += y;
         }
-        fine[x] = (j ? cdf[j - 1] : 0.0) + inc;
+        const double c = ((j ? cdf[j - 1] : 0.0) + inc) * scale;
+        fine[x] = c > 0.0 ? (uint64_t)fmin(c, 2.0 * kTwo53) : 0;  // (a NaN or infinite state: any table will do)
     }
 }
-// ... and guide[i] = first x with C_x > (i / N) S, i = 0..N (at most N - 1),
-// so that a shot with u in [i, i + 1) / N ends between guide[i] and
+// ... and guide[i] = first x with fine[x] > i 2^53 / N, i = 0..N (at most
+// N - 1), so that a shot with u in [i, i + 1) / N ends between guide[i] and
 // guide[i + 1]: about one table entry to read instead of a search of all.
-__global__ void __launch_bounds__(256) k_guide(const double* __restrict__ fine, uint32_t N, uint32_t* __restrict__ guide) {
-    const double step = fine[N - 1] / (double)N;  // (N is a power of two)
+__global__ void __launch_bounds__(256) k_guide(const uint64_t* __restrict__ fine, int n, uint32_t* __restrict__ guide) {
+    const uint32_t N = 1u << n;
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i <= N; i += gridDim.x * blockDim.x) {
-        const double t = (double)i * step;
+        const uint64_t t = (uint64_t)i << (53 - n);
         uint32_t lo = 0, hi = N - 1;
         while (lo < hi) {
             const uint32_t mid = (lo + hi) >> 1;
@@ -707,13 +830,14 @@ __global__ void __launch_bounds__(256) k_guide(const double* __restrict__ fine, 
     }
 }
 
-// One thread per four shots (one Philox block): three random 32-byte sectors
-// of L2 per shot (guide, table, table) against a warp's search and rescan of
-// 32 amplitudes.  QCrank read-out of 2^20 amplitudes, 4.9 10^7 shots: one warp
-// per shot took 41.4 ms.
+// One thread per four shots (one Philox block), all in integers (in FP64 the
+// compares alone were 1.1 ms of the example below): three random 32-byte
+// sectors of L2 per shot (guide, table, table) against a warp's search and
+// rescan of 32 amplitudes.  QCrank read-out of 2^20 amplitudes, 4.9 10^7 shots:
+// one warp per shot took 41.4 ms.
 template <typename V, bool PERM>
-__global__ void __launch_bounds__(256) k_sample_dense(const V* __restrict__ psi, const double* __restrict__ cdf,
-                                                      uint64_t nblocks, const double* __restrict__ fine,
+__global__ void __launch_bounds__(256) k_sample_dense(const V* __restrict__ psi, const double* __restrict__ cdf, int n,
+                                                      const uint64_t* __restrict__ fine,
                                                       const uint32_t* __restrict__ guide, uint64_t shots, uint64_t seed,
                                                       const double* __restrict__ u_in, uint64_t* __restrict__ out,
                                                       const QubitMap map) {
@@ -726,68 +850,65 @@ __global__ void __launch_bounds__(256) k_sample_dense(const V* __restrict__ psi,
         if constexpr (PERM) return psi[phys_index(qt, x)];
         else return psi[x];
     };
+    constexpr uint64_t D = (uint64_t)(kClear * kTwo53);
     const int lane = threadIdx.x & 31;
-    const double S = cdf[nblocks - 1], d = kClear * S, scale = (double)(nblocks << 5);
+    const uint64_t nblocks = 1ull << (n - 5);
     const uint64_t groups = (shots + 3) >> 2, stride = (uint64_t)gridDim.x * blockDim.x;
     for (uint64_t g0 = (uint64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); g0 < groups; g0 += stride) {
         const uint64_t g = g0 + lane;
         const int cnt = g >= groups ? 0 : (int)min((uint64_t)4, shots - 4 * g);  // this lane's shots
-        double t[4];
+        uint64_t w[4], x[4];  // u in units of 2^-53 (a caller's finer u: rounded down)
         uint32_t lo[4], hi[4];
         if (u_in) {
 #pragma unroll
-            for (int k = 0; k < 4; ++k) t[k] = k < cnt ? u_in[4 * g + k] : 0.0;
+            for (int k = 0; k < 4; ++k) w[k] = k < cnt ? (uint64_t)(u_in[4 * g + k] * kTwo53) : 0;
         } else {
             uint64_t c[4] = {g, 0, 0, 0};
             philox4x64_10(c, seed, 0);
 #pragma unroll
-            for (int k = 0; k < 4; ++k) t[k] = (double)(c[k] >> 11) * 0x1.0p-53;
+            for (int k = 0; k < 4; ++k) w[k] = c[k] >> 11;
         }
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            const uint32_t i = (uint32_t)(t[k] * scale);  // u < 1: i < N
+            const uint32_t i = (uint32_t)(w[k] >> (53 - n));  // u < 1: i < N
             lo[k] = guide[i];
             hi[k] = guide[i + 1];
-            t[k] *= S;
         }
         unsigned slow = 0;
-        uint64_t x[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             uint32_t a = lo[k], b = hi[k];
             while (a < b) {
                 const uint32_t mid = (a + b) >> 1;
-                if (fine[mid] > t[k]) b = mid;
+                if (fine[mid] > w[k]) b = mid;
                 else a = mid + 1;
             }
             x[k] = a;
-            const double prev = a ? fine[a - 1] : -1.0;
-            // (a NaN total or table fails the compares and goes the slow way)
-            if (k < cnt && !(fine[a] > t[k] + d && (prev < t[k] - d || a == 0))) slow |= 1u << k;
+            if (k < cnt && !(fine[a] > w[k] + D && (a == 0 || fine[a - 1] + D < w[k]))) slow |= 1u << k;
         }
         for (unsigned m = __ballot_sync(0xffffffffu, slow != 0); m; m &= m - 1) {
             const int src = __ffs(m) - 1;
             const unsigned ks = __shfl_sync(0xffffffffu, slow, src);
+            const uint64_t gs = __shfl_sync(0xffffffffu, g, src);
+            const double S = cdf[nblocks - 1];
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 if (!((ks >> k) & 1)) continue;
-                const double ts = __shfl_sync(0xffffffffu, t[k], src);
-                const uint64_t j = warp_find_block(cdf, nblocks, ts, lane);
-                const uint64_t r = warp_sample<V>(amp, 5, cdf, j, S, ts, lane);
+                const uint64_t ws = __shfl_sync(0xffffffffu, w[k], src);
+                const double t = (u_in ? u_in[4 * gs + k] : (double)ws * 0x1.0p-53) * S;
+                const uint64_t r = warp_sample<V>(amp, 5, cdf, warp_find_block(cdf, nblocks, t, lane), S, t, lane);
                 if (lane == src) x[k] = r;
             }
         }
-        if (cnt == 4) {
+        if (cnt == 4 && ((uintptr_t)out & 15) == 0) {
             ulonglong2* o = (ulonglong2*)(out + 4 * g);
-            if (((uintptr_t)out & 15) == 0) {
-                o[0] = make_ulonglong2(x[0], x[1]);
-                o[1] = make_ulonglong2(x[2], x[3]);
-                continue;
-            }
-        }
+            o[0] = make_ulonglong2(x[0], x[1]);
+            o[1] = make_ulonglong2(x[2], x[3]);
+        } else {
 #pragma unroll
-        for (int k = 0; k < 4; ++k)
-            if (k < cnt) out[4 * g + k] = x[k];
+            for (int k = 0; k < 4; ++k)
+                if (k < cnt) out[4 * g + k] = x[k];
+        }
     }
 }
 
@@ -888,7 +1009,7 @@ static int logical_block_cdf(sv_state* h, int blog, double** cdf_out, int64_t* n
 // [chunk totals: nch][bit sums: 10 nb, when asked for][quarter totals: 4 nb,
 // when asked for and the kernel has them; else *quart_out = nullptr].
 static int block_stats(sv_state* h, bool want_bits, double** tot_out, double** cdf_out, double** bits_out,
-                       int* blog_out, int64_t* nb_out, int blog_cap = kBlogMax, double** quart_out = nullptr) {
+                       int* blog_out, int64_t* nb_out, int blog_cap = kBlogMax, float2** quart_out = nullptr) {
     int blog;
     const size_t nb = nblocks_of(h->n, &blog, blog_cap);
     const size_t nch = (nb + kScanCh - 1) / kScanCh;
@@ -900,7 +1021,7 @@ static int block_stats(sv_state* h, bool want_bits, double** tot_out, double** c
     double* cdf = tot + nb;
     double* chunks = cdf + nb;
     double* bits = want_bits ? chunks + nch + 64 : nullptr;
-    double* quart = quarters ? bits + 10 * nb : nullptr;
+    float2* quart = quarters ? (float2*)(bits + 10 * nb) : nullptr;
     if (quart_out) *quart_out = quart;
     const unsigned g = (unsigned)((nb * 32 + 255) / 256);
     count_launch();
@@ -1017,28 +1138,27 @@ template <typename V, bool PERM>
 static void dense_t(sv_state* h, const double* cdf, int64_t nb, uint64_t shots, uint64_t seed, const double* dev_u,
                     uint64_t* dev_out, const QubitMap& map) {
     const V* a = (const V*)h->amps;
-    const uint32_t N = 1u << h->n;
-    double* fine = (double*)h->fine.ptr;
-    uint32_t* guide = (uint32_t*)(fine + N);
+    uint64_t* fine = (uint64_t*)h->fine.ptr;
+    uint32_t* guide = (uint32_t*)(fine + (1ull << h->n));
     const unsigned cap = (unsigned)sms() * 8;
     const unsigned gf = (unsigned)std::min<uint64_t>(((uint64_t)nb * 32 + 255) / 256, cap);
     const unsigned gs = (unsigned)std::min<uint64_t>(((shots + 3) / 4 + 255) / 256, cap);
     count_launch(3);
     k_fine_cdf<V, PERM><<<gf, 256, 0, h->stream>>>(a, cdf, (uint64_t)nb, fine, map);
-    k_guide<<<gf, 256, 0, h->stream>>>(fine, N, guide);
-    k_sample_dense<V, PERM><<<gs, 256, 0, h->stream>>>(a, cdf, (uint64_t)nb, fine, guide, shots, seed, dev_u, dev_out,
-                                                      map);
+    k_guide<<<gf, 256, 0, h->stream>>>(fine, h->n, guide);
+    k_sample_dense<V, PERM><<<gs, 256, 0, h->stream>>>(a, cdf, h->n, fine, guide, shots, seed, dev_u, dev_out, map);
 }
 
 // Shots from a block CDF; logical = the CDF is in logical order (relabelled
-// state) and the outcomes come out as logical indices.  quart: see k_sample.
+// state) and the outcomes come out as logical indices.  quart: quarter totals
+// of the blocks (see k_sample_quarter) where block_stats has them.
 static cudaError_t launch_sample(sv_state* h, int blog, const double* cdf, int64_t nb, uint64_t shots,
                                  uint64_t seed, const double* dev_u, uint64_t* dev_out, bool logical = false,
-                                 const double* quart = nullptr) {
+                                 const float2* quart = nullptr) {
     const QubitMap map = qubit_map(h);
     // (without memory for the table the shots go one warp at a time)
     if (dense_shots(h->n, blog, shots) &&
-        ensure_scratch(&h->fine, (sizeof(double) << h->n) + sizeof(uint32_t) * ((1ull << h->n) + 1), h->stream) == SV_OK) {
+        ensure_scratch(&h->fine, (sizeof(uint64_t) << h->n) + sizeof(uint32_t) * ((1ull << h->n) + 1), h->stream) == SV_OK) {
         if (h->dtype == SV_C64) {
             if (logical) dense_t<float2, true>(h, cdf, nb, shots, seed, dev_u, dev_out, map);
             else dense_t<float2, false>(h, cdf, nb, shots, seed, dev_u, dev_out, map);
@@ -1048,20 +1168,29 @@ static cudaError_t launch_sample(sv_state* h, int blog, const double* cdf, int64
         }
         return cudaGetLastError();
     }
+    const uint64_t n = (uint64_t)nb;
+    if (quart && !dev_u && !logical) {
+        // shots per warp: as many as leave 16 warps per SM
+        const int G = (int)std::max<uint64_t>(1, std::min<uint64_t>(32, shots / ((uint64_t)sms() * 16)));
+        const uint64_t warps = (shots + G - 1) / G;
+        const unsigned gq = (unsigned)std::min<uint64_t>((warps + 7) / 8, (uint64_t)sms() * 8);
+        count_launch();
+        k_sample_quarter<<<gq, 256, 0, h->stream>>>((const float2*)h->amps, cdf, n, quart, G, shots, seed, dev_out);
+        return cudaGetLastError();
+    }
     uint64_t g = (shots * 32 + 255) / 256;
     const uint64_t cap = (uint64_t)sms() * 16;
     if (g > cap) g = cap;
     count_launch();
     const unsigned gg = (unsigned)g;
-    const uint64_t n = (uint64_t)nb;
     if (h->dtype == SV_C64) {
         const float2* a = (const float2*)h->amps;
-        if (logical) k_sample<float2, true><<<gg, 256, 0, h->stream>>>(a, blog, cdf, n, nullptr, shots, seed, dev_u, dev_out, map);
-        else k_sample<float2, false><<<gg, 256, 0, h->stream>>>(a, blog, cdf, n, quart, shots, seed, dev_u, dev_out, map);
+        if (logical) k_sample<float2, true><<<gg, 256, 0, h->stream>>>(a, blog, cdf, n, shots, seed, dev_u, dev_out, map);
+        else k_sample<float2, false><<<gg, 256, 0, h->stream>>>(a, blog, cdf, n, shots, seed, dev_u, dev_out, map);
     } else {
         const double2* a = (const double2*)h->amps;
-        if (logical) k_sample<double2, true><<<gg, 256, 0, h->stream>>>(a, blog, cdf, n, nullptr, shots, seed, dev_u, dev_out, map);
-        else k_sample<double2, false><<<gg, 256, 0, h->stream>>>(a, blog, cdf, n, nullptr, shots, seed, dev_u, dev_out, map);
+        if (logical) k_sample<double2, true><<<gg, 256, 0, h->stream>>>(a, blog, cdf, n, shots, seed, dev_u, dev_out, map);
+        else k_sample<double2, false><<<gg, 256, 0, h->stream>>>(a, blog, cdf, n, shots, seed, dev_u, dev_out, map);
     }
     return cudaGetLastError();
 }
@@ -1080,21 +1209,24 @@ static int sample_logical(sv_state* h, int blog, uint64_t shots, uint64_t seed, 
 
 // Shots and <Z_i> from ONE pass over the state (either output may be NULL).
 int measure_readout(sv_state* h, uint64_t shots, uint64_t seed, uint64_t* dev_samples, double* dev_expz) {
-    double *tot, *cdf, *bits, *quart = nullptr;
+    double *tot, *cdf, *bits;
+    float2* quart = nullptr;
     int blog;
     int64_t nb;
     const bool here = dev_samples && shots && !h->permuted;  // shots drawn from these blocks
     int rc = block_stats(h, dev_expz != nullptr, &tot, &cdf, &bits, &blog, &nb, kBlogMax, here ? &quart : nullptr);
     if (rc) return rc;
     if (dev_expz) {
-        // chunk partials, then (relabelled qubits) the physical-bit values
-        rc = ensure_scratch(&h->perm_tmp, sizeof(double) * (2 * 64 * kExpzChunks + 64), h->stream);
+        // CTA partials, then (relabelled qubits) the physical-bit values
+        const ExpzItem I = expz_item(0, (uint64_t)nb, h->n, blog, 0, h->dtype, (uint64_t)nb);
+        const size_t np = (size_t)kExpzSlots << I.lg;
+        rc = ensure_scratch(&h->perm_tmp, sizeof(double) * (np + 64), h->stream);
         if (rc) return rc;
         double* part = (double*)h->perm_tmp.ptr;
-        double* ez = h->permuted ? part + 2 * 64 * kExpzChunks : dev_expz;
+        double* ez = h->permuted ? part + np : dev_expz;
         count_launch(2);
-        k_expz_blocks<<<dim3(h->n, kExpzChunks), 256, 0, h->stream>>>(tot, bits, (uint64_t)nb, blog, part);
-        k_expz_final<<<1, 64, 0, h->stream>>>(part, h->n, ez);
+        k_expz_part<<<1u << I.lg, 256, 0, h->stream>>>(tot, bits, nullptr, I, part);
+        k_expz_sum<<<(unsigned)h->n, 32, 0, h->stream>>>(part, nullptr, I, 1 << I.lg, ez);
         if (h->permuted) {
             count_launch();
             k_logical_expz<<<1, 64, 0, h->stream>>>(ez, dev_expz, qubit_map(h));
@@ -1110,6 +1242,47 @@ int measure_readout(sv_state* h, uint64_t shots, uint64_t seed, uint64_t* dev_sa
         if (e != cudaSuccess) return cuda_fail(e, "read-out");
     }
     return SV_OK;
+}
+
+// <Z_i> of C states that lie one after the other from base (state c: n[c]
+// qubits, at least kBlogMax, at amplitude offs[c]), row c of dev_out (nmax
+// apart): three launches for all of them, enqueued on st.
+int measure_expz_many(int dtype, const void* base, int C, const uint64_t* offs, const int* n, uint64_t amps,
+                      double* const* rows, cudaStream_t st, std::vector<void*>* pinned) {
+    const uint64_t nb = amps >> kBlogMax;
+    std::vector<ExpzItem> items;
+    int lg = 0, nmax = 0;
+    for (int c = 0; c < C; ++c) {
+        ExpzItem I = expz_item(offs[c] >> kBlogMax, 1ull << (n[c] - kBlogMax), n[c], kBlogMax,
+                               (uint64_t)(rows[c] - rows[0]), dtype, nb);
+        nmax = std::max(nmax, n[c]);
+        lg = std::max(lg, I.lg);
+        items.push_back(I);
+    }
+    const size_t ib = (sizeof(ExpzItem) * (size_t)C + 15) & ~(size_t)15, npart = ((size_t)kExpzSlots * C) << lg;
+    void *dev = nullptr, *pin = nullptr;
+    cudaError_t e = cudaMallocAsync(&dev, ib + sizeof(double) * (11 * nb + npart), st);
+    if (e == cudaSuccess) e = cudaMallocHost(&pin, ib);
+    if (pin) pinned->push_back(pin);
+    if (e != cudaSuccess) {
+        if (dev) cudaFreeAsync(dev, st);
+        cudaGetLastError();
+        return set_error(SV_ENOMEM, "read-out scratch of the wave");
+    }
+    double* tot = (double*)((char*)dev + ib);
+    double* bits = tot + nb;
+    double* part = bits + 10 * nb;
+    memcpy(pin, items.data(), sizeof(ExpzItem) * (size_t)C);
+    e = cudaMemcpyAsync(dev, pin, ib, cudaMemcpyHostToDevice, st);
+    const unsigned g = (unsigned)((nb * 32 + 255) / 256);
+    count_launch(3);
+    if (dtype == SV_C64) k_block_stats<float2><<<g, 256, 0, st>>>((const float2*)base, kBlogMax, nb, tot, bits, nullptr);
+    else k_block_stats<double2><<<g, 256, 0, st>>>((const double2*)base, kBlogMax, nb, tot, bits, nullptr);
+    k_expz_part<<<dim3(1u << lg, (unsigned)C), 256, 0, st>>>(tot, bits, (const ExpzItem*)dev, ExpzItem{}, part);
+    k_expz_sum<<<dim3((unsigned)nmax, (unsigned)C), 32, 0, st>>>(part, (const ExpzItem*)dev, ExpzItem{}, 1 << lg, rows[0]);
+    if (e == cudaSuccess) e = cudaGetLastError();
+    cudaFreeAsync(dev, st);
+    return e == cudaSuccess ? SV_OK : cuda_fail(e, "read-out of the wave");
 }
 
 int measure_expect_z(sv_state* h, double* dev_out) { return measure_readout(h, 0, 0, nullptr, dev_out); }
@@ -1219,11 +1392,10 @@ extern "C" int sv_sample_uniforms_noalloc(const void* dev_amps, int n, sv_dtype 
     if (gs > cap) gs = cap;
     count_launch();
     if (dt == SV_C64)
-        k_sample<float2, false><<<(unsigned)gs, 256, 0, st>>>((const float2*)dev_amps, blog, bs, (uint64_t)nb, nullptr,
+        k_sample<float2, false><<<(unsigned)gs, 256, 0, st>>>((const float2*)dev_amps, blog, bs, (uint64_t)nb,
                                                              shots, 0, dev_u, dev_out, QubitMap{});
     else
-        k_sample<double2, false><<<(unsigned)gs, 256, 0, st>>>((const double2*)dev_amps, blog, bs, (uint64_t)nb,
-                                                              nullptr, shots, 0, dev_u, dev_out, QubitMap{});
+        k_sample<double2, false><<<(unsigned)gs, 256, 0, st>>>((const double2*)dev_amps, blog, bs, (uint64_t)nb, shots, 0, dev_u, dev_out, QubitMap{});
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "sv_sample_uniforms_noalloc");
     return SV_OK;
