@@ -734,6 +734,7 @@ PassLayout pass_layout(int dtype, const PassDev& P) {
 // returns.
 constexpr int kMaxSlots = 4;
 constexpr uint32_t kTmaWaitLimit = 1u << 22;
+constexpr int kMaxDynSmemTma = 223 * 1024;  // 227 KB per block less this kernel's static variables (3.5 KB)
 
 struct RingLayout {
     int slots;
@@ -830,7 +831,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_rpass_tma(int n, const PassDev* __r
         V* tile = (V*)(smem + (size_t)s * lay.tile_bytes);
         if (P.ndiag) fold_diags<R>(P, stage, fold, dofs, t);
         TcCtx T0{0u, nullptr, nullptr, err, 0u, nullptr, nullptr};  // (TMA-fed passes carry no tensor-core blocks)
-        InterpOps<false>::tile<V, R, RB>(v, tile, P, stage, fold, Lg, nullptr, T0);
+        InterpOps<false, RB>::template tile<V, R, RB>(v, tile, P, stage, fold, Lg, nullptr, T0);
         if (P.scale != 1.0) {
             const R sc = (R)P.scale;
 #pragma unroll
@@ -840,6 +841,8 @@ __global__ void __launch_bounds__(MAXT, 1) k_rpass_tma(int n, const PassDev* __r
             }
         }
         __syncthreads();
+#pragma unroll
+        for (int b = 0; b < RB; ++b) Lg.sbit[b] = swz<V>(P.fmask[b]);
         reg_write<V, RB>(v, tile, Lg);
         tc::fence_proxy_async();
         __syncthreads();
@@ -887,7 +890,7 @@ PassLayout rpass_layout(int dtype, const PassDev& P, bool single) {
         // for its whole (persistent) run: ask for enough shared memory that no
         // more CTAs share an SM than its 512 columns serve, so no allocation
         // ever waits for a co-resident CTA to finish
-        const int groups = std::max(1, (1 << (m - reg_bits(dtype))) >> 7);
+        const int groups = std::max(1, (1 << (m - P.rb)) >> 7);
         const int fit = std::max(1, 4 / groups);
         const int need = kSmemPerSm / (fit + 1) + 1024;
         if (lay.total < need) lay.total = need;
@@ -1208,6 +1211,16 @@ static cudaError_t pass_t(sv_state* h, const void* blob_dev, const PlanBlob& blo
     return cudaGetLastError();
 }
 
+// Whether a pass may start before the previous one has finished: its CTAs then
+// find idle SMs (at most one for every two), or fill the GPU anyway and take
+// the places of the previous pass's as they end.  In between they would crowd
+// onto the few SMs the previous pass left idle (20 qubits, 128 CTAs: passes a
+// fifth slower).
+bool pdl_pays(int pass, uint64_t grid, int per_sm) {
+    const uint64_t sms = (uint64_t)num_sms();
+    return pass > 0 && (2 * grid <= sms || grid == sms * per_sm);
+}
+
 template <typename R, int RB, int MAXT, int MINB, bool TC>
 static cudaError_t rpass_t(sv_state* h, const void* blob_dev, const PlanBlob& blob, int pass) {
     using V = typename CT<R>::V;
@@ -1236,9 +1249,21 @@ static cudaError_t rpass_t(sv_state* h, const void* blob_dev, const PlanBlob& bl
     if (grid > ntiles) grid = ntiles;
     const unsigned char* b = (const unsigned char*)blob_dev;
     count_launch();
-    k_rpass<R, RB, MAXT, MINB, TC><<<(unsigned)grid, threads, lay.total, h->stream>>>(
-        (V*)h->amps, h->n, (const PassDev*)(b + blob.pass_off) + pass, b, lay, (int*)h->err.ptr);
-    return cudaGetLastError();
+    // may start before the previous pass has finished (rpass_body waits for it
+    // before it touches the state); not with tensor-core blocks, whose TMEM the
+    // previous pass's CTAs may still hold
+    cudaLaunchAttribute pdl{};
+    pdl.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    pdl.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = (size_t)lay.total;
+    cfg.stream = h->stream;
+    cfg.attrs = &pdl;
+    cfg.numAttrs = !TC && pdl_pays(pass, grid, per_sm) ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, k_rpass<R, RB, MAXT, MINB, TC>, (V*)h->amps, h->n,
+                              (const PassDev*)(b + blob.pass_off) + pass, b, lay, (int*)h->err.ptr);
 }
 
 template <typename R, int RB, bool TC>
@@ -1252,6 +1277,8 @@ static cudaError_t rpass_tc(sv_state* h, const void* blob_dev, const PlanBlob& b
 template <typename R, int RB>
 static cudaError_t rpass_any(sv_state* h, const void* blob_dev, const PlanBlob& blob, int pass, int m) {
     const PassDev* pdh = (const PassDev*)(blob.bytes.data() + blob.pass_off) + pass;
+    // (plans with small_reg_bits have at most 256 threads)
+    if (pdh->rb == RB - 1) return rpass_t<R, RB - 1, 256, 3, false>(h, blob_dev, blob, pass);
     if constexpr (sizeof(R) == 4 && RB == 5)
         if (pdh->tc_k > 0) return rpass_tc<R, RB, true>(h, blob_dev, blob, pass, m);
     return rpass_tc<R, RB, false>(h, blob_dev, blob, pass, m);
@@ -1373,15 +1400,15 @@ __global__ void __launch_bounds__(256, MUX ? 1 : 2) k_wave(typename CT<R>::V* __
             __syncthreads();
             for (uint64_t t = I.lo; t < I.hi; ++t) {
                 const uint64_t b = table_base(tbase, t, P.L);
-                rissue_tile(tile, psi, b, rowoff, P.L);
+                rissue_tile<V, RB>(tile, psi, b, rowoff, P.L);
                 cp_async_commit();
                 cp_async_wait_group<0>();
                 __syncthreads();
                 if (P.ndiag) fold_diags<R>(P, stage, fold, dofs, t);
-                InterpOps<false>::tile<V, R, RB>(v, tile, P, stage, fold, Lg, sizeof(R) == 8 ? ttab : nullptr, T0);
-                InterpOps<false>::finish<V, R, RB>(v, tile, P, Lg, T0);
+                InterpOps<false, RB>::template tile<V, R, RB>(v, tile, P, stage, fold, Lg, sizeof(R) == 8 ? ttab : nullptr, T0);
+                InterpOps<false, RB>::template finish<V, R, RB>(v, tile, P, Lg, T0);
                 __syncthreads();
-                rstore_tile(tile, psi, b, rowoff, P.L);
+                rstore_tile<V, RB>(tile, psi, b, rowoff, P.L);
                 __syncthreads();
             }
         }
@@ -1502,7 +1529,7 @@ int box_rows(const PassDev& P) {
 // The ring: as many slots (2..4) as keep the most warps per SM busy.
 static bool ring_layout(int dtype, const PassDev& P, RingLayout* out, int* ctas_per_sm) {
     const size_t csz = dtype == SV_C64 ? 8 : 16;
-    const int m = P.m, nrows = 1 << (m - P.L), threads = 1 << (m - reg_bits(dtype));
+    const int m = P.m, nrows = 1 << (m - P.L), threads = 1 << (m - P.rb);
     RingLayout lay;
     memset(&lay, 0, sizeof(lay));
     lay.tile_bytes = (int)(csz << m);
@@ -1514,7 +1541,7 @@ static bool ring_layout(int dtype, const PassDev& P, RingLayout* out, int* ctas_
     int best_score = -1;
     for (int S = kMaxSlots; S >= 2; --S) {
         const int total = S * lay.tile_bytes + rest;
-        if (total > kMaxDynSmem) continue;
+        if (total > kMaxDynSmemTma) continue;
         const int ctas = std::max(1, std::min(8, (228 * 1024) / (total + 1024)));
         const int warps = std::min(16, ctas * threads / 32);
         const int score = warps * 8 + S;

@@ -100,11 +100,11 @@ bool build_wave(int dtype, const std::vector<const Plan*>& plans, WaveHost* w,
                 const std::vector<const PlanBlob*>* blobs) {
     if (blobs) merge_blobs(*blobs, &w->blob);
     else serialise_plans(plans, &w->blob);
-    const int RB = reg_bits(dtype);
     const unsigned char* b = w->blob.bytes.data();
     const PassDev* pds = (const PassDev*)(b + w->blob.pass_off);
+    const int RB = reg_bits(dtype);
     for (int p = 0; p < w->blob.npasses; ++p)
-        if (!(pds[p].rmode == kRmodeMux || (pds[p].rmode == 1 && pds[p].m - RB == 8 && pds[p].tc_k == 0)))
+        if (!(pds[p].rmode == kRmodeMux || (pds[p].rmode == 1 && pds[p].rb == RB && pds[p].m - RB == 8 && pds[p].tc_k == 0)))
             return false;
     const int C = (int)plans.size();
     std::vector<int> first(C + 1, 0);
@@ -307,6 +307,15 @@ extern "C" int sv_batch_run(int C, const int* n_qubits, const int64_t* gate_offs
         bad[c] = canonicalise(n, gates + gate_offsets[c], (size_t)gate_counts[c], &cg[c], &b) != SV_OK;
         if (bad[c] || n <= small_limit(dt) || !host_plans) return;
         PlanOptions po = resolve_options(n, dt, opt);
+        po.fold_perms = true;  // (never compiled)
+        if (po.rb != reg_bits(dt)) {
+            // the wave kernel holds the wide register count: a wave has warps
+            // enough, and fewer passes and remaps (256 20-qubit ansatz circuits:
+            // 62.9 ms, with 2^4 amplitudes per thread 67.8 ms)
+            po.rb = reg_bits(dt);
+            po.k_max = dt == SV_C64 ? kMaxK : 4;
+            po.tile_m = std::min(n, po.rb + 8);
+        }
         po.tc_auto = 0;  // the wave kernel runs the interpreting pass body, without tensor-core blocks
         if (po.tensor == 0) po.tensor = -1;
         std::vector<CGate>& g = cg[c];
@@ -628,6 +637,9 @@ extern "C" int sv_selftest_wave_timeout(unsigned limit, int* host_status) {
     if (canonicalise(n, g.data(), g.size(), &cg, &bad) != SV_OK) return set_error(SV_EINVAL, "internal: circuit");
     PlanOptions po = resolve_options(n, SV_C64, nullptr);
     po.tc_auto = 0;
+    po.rb = reg_bits(SV_C64);
+    po.k_max = kMaxK;
+    po.tile_m = po.rb + 8;  // 256 threads
     Plan plan;
     plan_greedy(n, SV_C64, cg, po, &plan);
     WaveHost w;

@@ -277,6 +277,7 @@ bool plan_learned(int n, int dtype, const std::vector<CGate>& gates, const std::
     out->no_register_passes = false;
     out->use_tma = false;
     out->jit = base.jit;
+    out->rb = base.rb;
     out->passes.clear();
     for (auto it = chain.rbegin(); it != chain.rend(); ++it) {
         HostPass hp = std::move(nodes[*it].hp);
@@ -360,7 +361,8 @@ extern "C" int sv_cost_model_choose(int n, sv_dtype dt, const sv_gate* gates, si
     size_t bad = 0;
     if (canonicalise(n, gates, count, &cg, &bad) != SV_OK)
         return set_error(SV_EINVAL, "invalid gate record at index " + std::to_string(bad));
-    const PlanOptions base = resolve_options(n, dt, nullptr);
+    PlanOptions base = resolve_options(n, dt, nullptr);
+    base.rb = reg_bits(dt);  // the candidates are compiled passes
     std::vector<PlanOptions> ranked;
     std::vector<double> rms;
     if (!rank_options(n, dt, cg, nullptr, base, &ranked, &rms)) return set_error(SV_EINVAL, "no cost model loaded");
@@ -387,7 +389,8 @@ extern "C" int sv_cost_model_judged(int n, sv_dtype dt, const sv_gate* gates, si
                                     double* measured_ms) {
     if (!out || (count && !gates)) return set_error(SV_EINVAL, "bad arguments");
     uint64_t key = fnv1a(gates, count * sizeof(sv_gate), 1469598103934665603ull);
-    const PlanOptions base = resolve_options(n, dt, nullptr);
+    PlanOptions base = resolve_options(n, dt, nullptr);
+    base.rb = reg_bits(dt);  // the candidates are compiled passes
     const int meta[3] = {n, (int)dt, base.tensor};
     key = fnv1a(meta, sizeof(meta), key);
     std::lock_guard<std::mutex> lk(g_mu);

@@ -21,30 +21,45 @@ enum OpKind { OP_DENSE = 0, OP_DIAG = 1, OP_GATES = 2, OP_REMAP = 3, OP_DENSE_TC
 __host__ __device__ inline int pass_max_threads(int tb) { return tb <= 7 ? 128 : (tb == 8 ? 256 : 512); }
 __host__ __device__ inline int pass_min_blocks(int tb) { return tb <= 8 ? 2 : 1; }
 
-// Register-resident passes: each thread holds 2^kRegBits amplitudes of the
-// tile in registers; the other m - kRegBits tile bits index the thread.
+// Register-resident passes: each thread holds 2^rb amplitudes of the tile in
+// registers; the other m - rb tile bits index the thread.  rb = reg_bits (64
+// registers of amplitudes) for compiled passes and whatever the caller asks
+// for by width; small_reg_bits (32 registers) where the interpreting kernel
+// runs the plan (PlanOptions::rb says when).
 __host__ __device__ inline int reg_bits(int dtype) { return dtype == 0 ? 5 : 4; }  // 0: complex64
+__host__ __device__ inline int small_reg_bits(int dtype) { return dtype == 0 ? 4 : 3; }
 constexpr int kRegDenseMaxK = 3;  // dense blocks in registers (wider ones run as gate sequences)
 constexpr int kStageCap = 48 * 1024;  // bytes of a pass region staged in shared memory
 constexpr int kStageCapTc = 100 * 1024;  // the same for a pass with tensor-core blocks
 
 // Gate-sequence block records (positions are block-local bits, data offsets
 // index the op's own complex values).
-enum GateRecKind { GR_U = 0, GR_UR = 1, GR_DT = 2, GR_CX = 3, GR_SWAP = 4, GR_H = 5, GR_HD = 6, GR_URS = 7 };
+enum GateRecKind { GR_U = 0, GR_UR = 1, GR_DT = 2, GR_CX = 3, GR_SWAP = 4, GR_H = 5, GR_HD = 6, GR_URS = 7, GR_DTS = 8, GR_RS = 9 };
 // GR_DT: a = mask of the positions its entries depend on (entry j equals
 // entry j & a), b = mask of the entries that differ from 1 (register passes).
 // GR_HD (register passes only): GR_H on position a followed by the phase table
 // at off with entry mask b (one dispatch for the pair).
-// GR_URS (register passes only): a rotation [[c, -s], [s, c]] on position a
-// without its larger factor: [[1, -t], [t, 1]] with t = s / c (b = 0) or
-// [[t, -1], [1, t]] with t = c / s (b = 1), t at off; the factor joins
-// PassDev::scale like GR_H's.
+// GR_URS (register passes only): a rotation [[c, -s], [s, c]] on position a as
+// [[1, -t], [t, 1]], t = s / c; (t, t) and (-t, -t) at off, the factor c joins
+// PassDev::scale like GR_H's.  One form for every angle, so circuits of one
+// shape share their compiled passes; a rotation with |c| < kMinDeferredCos stays
+// a GR_UR (t would use up the range the deferred factors may take).
+// GR_DTS, GR_RS (complex128 register passes): a phase table without its
+// cosines and a rotation of amplitudes that lack them.  e^{i f} = cos f (1 + i
+// tan f): GR_DTS applies 1 + i tan f_j (2^r real tangents at off, b = mask of
+// the entries that differ from 1), two FP64 operations per amplitude instead of
+// four, and leaves register j short of a real factor s_j known to the planner.
+// GR_RS rotates such registers, v_j += c_j v_j' for the partner j' = j ^ 2^a (2^r
+// reals c at off, the tangent times s_j' / s_j), which costs what GR_URS does.
+// The last table before the block's end, or before a record that needs equal
+// factors, is a GR_DT whose entries include s_j.
 // GR_H (register passes only): the Hadamard without its 1/sqrt(2), a + b and
 // a - b; the pass multiplies its amplitudes by the product of the dropped
 // factors once, when it writes them back (PassDev::scale).
 struct GateRec {
     int kind, a, b, off;
 };
+constexpr double kMinDeferredCos = 0x1p-10;
 constexpr int kMaxGateRecs = 64;     // records per gate-sequence op
 constexpr int kMaxGateData = 768;    // complex values per gate-sequence op
 
@@ -69,7 +84,8 @@ struct OpDev {
     int ndata;     // gates: complex values at mat_off
     int ord;       // register passes, diag: ordinal of the run within the pass
     float tc_scale;  // OP_DENSE_TC: factor applied to the registers before the FP16 split
-    int pad[3];
+    int wmask[kMaxK];  // remap: tile positions register bit b flips in the layout written back (folded permutations)
+    int pad[2];
 };
 static_assert(sizeof(OpDev) % 16 == 0, "OpDev array must keep 16-byte alignment");
 
@@ -104,6 +120,9 @@ struct PassDev {
     int rmode;           // register-resident pass (region in the register format): 1 fed by
                          // cp.async copies, 2 by TMA tensor copies; 0: shared-memory kernel;
                          // kRmodeMux: multiplexor pass
+    int rb;              // register passes: 2^rb amplitudes per thread
+    int folded;          // register passes: some wmask or fmask is not the layout's own
+    int fmask[kMaxK];    // register passes: wmask of the final write-back
     int ndiag;           // register passes: diagonal runs (each folded once per tile)
     int nops;            // ops in the pass's region
     int region_off;      // byte offset of the region in the blob

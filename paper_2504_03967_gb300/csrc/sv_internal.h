@@ -49,11 +49,10 @@ int canonicalise(int n, const sv_gate* g, size_t count, std::vector<CGate>* out,
 // 2^L amplitudes is contiguous), applies its ops in shared memory and writes
 // the tile back: one HBM read and one write of the state per pass.
 // ---------------------------------------------------------------------------
-// Widest gate-sequence block: its 2^k amplitudes per thread stay in
-// registers (64 registers of data at the bound, for both dtypes).  The
+// Widest gate-sequence block: the plan's rb (its 2^k amplitudes per thread stay
+// in registers, 64 registers of data at the bound, for both dtypes).  The
 // shared-memory pass kernel, which holds more state per thread, takes one
 // qubit less and runs wider blocks from their dense matrix.
-inline int max_gates_k(int dtype) { return dtype == SV_C64 ? 5 : 4; }
 inline int smem_gates_max_k(int dtype) { return dtype == SV_C64 ? 4 : 3; }
 // Tile rows: qubits 0..L-1 are always tile qubits, so a tile is made of rows
 // of 2^L contiguous amplitudes, 128 bytes (the TMA-fed kernel's tensor-map
@@ -161,6 +160,8 @@ struct Plan {
     bool no_register_passes = false;
     bool use_tma = false;  // register passes move tiles with TMA tensor copies
     int jit = 0;           // PlanOptions::jit
+    int rb = 5;            // PlanOptions::rb
+    bool fold_perms = false;  // PlanOptions::fold_perms
     std::vector<Mux> muxes;
 };
 
@@ -182,11 +183,18 @@ struct PlanOptions {
     double drop_phase_below = 0.0;  // approximation: smaller P/RZ/CP angles are dropped
     int mux = 0;          // multiplexor recognition: 0 long runs, 1 any run of 4+ gates, -1 off
     int jit = 0;          // run-time compiled register passes: 0 on repeat, 1 always, -1 never
+    int rb = 5;           // register passes hold 2^rb amplitudes per thread (see resolve_options)
+    bool fold_perms = false;  // the interpreting kernel will run the plan: CX and SWAP gates a block can end
+                              // with join the addresses the block's registers are written back to
     int tc_auto = 0;      // tensor-core dense blocks where their estimated cost is below the gate sequence's
 };
 // The approximation for negligible rotations: the gates kept.
 void drop_small_phases(std::vector<CGate>* g, double eps);
 
+// jit = 0 compiles only for states of at least this many qubits: below it a
+// pass takes tens of microseconds, and the compile (about a second) would not
+// pay back.
+constexpr int kJitAutoMinQubits = 22;
 PlanOptions resolve_options(int n, int dtype, const sv_options* opt);
 // GK_MUX gates index muxes (may be null when there are none); the plan keeps
 // a copy of the multiplexors its passes use.
@@ -370,6 +378,7 @@ PassLayout rpass_layout(int dtype, const PassDev& P, bool single = false);  // s
 // per 128 threads, for passes with tensor-core blocks).
 int resident_ctas(int threads, int regs, int smem);
 int num_sms_pub();
+bool pdl_pays(int pass, uint64_t grid, int per_sm);
 // Run-time compiled register passes (sv_jit.cpp).  jit_prepare: per pass of
 // the blob, the compiled kernel ready for it (else nullptr); policy 1
 // compiles missing ones now, 0 once a structure is seen a second time on a

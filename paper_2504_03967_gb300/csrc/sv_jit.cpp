@@ -54,8 +54,7 @@ struct Driver {
     CUresult (*set_attr)(CUfunction, CUfunction_attribute, int) = nullptr;
     CUresult (*occupancy)(int*, CUfunction, int, size_t) = nullptr;
     CUresult (*get_attr)(int*, CUfunction_attribute, CUfunction) = nullptr;
-    CUresult (*launch)(CUfunction, unsigned, unsigned, unsigned, unsigned, unsigned, unsigned, unsigned, CUstream,
-                       void**, void**) = nullptr;
+    CUresult (*launch)(const CUlaunchConfig*, CUfunction, void**, void**) = nullptr;
 };
 
 template <typename F> bool sym(void* lib, const char* name, F* out) {
@@ -99,7 +98,7 @@ const Driver& driver() {
         d.ok = entry("cuModuleLoadData", &d.module_load) && entry("cuModuleGetFunction", &d.get_function) &&
                entry("cuFuncSetAttribute", &d.set_attr) &&
                entry("cuOccupancyMaxActiveBlocksPerMultiprocessor", &d.occupancy) &&
-               entry("cuFuncGetAttribute", &d.get_attr) && entry("cuLaunchKernel", &d.launch);
+               entry("cuFuncGetAttribute", &d.get_attr) && entry("cuLaunchKernelEx", &d.launch);
     });
     return d;
 }
@@ -223,14 +222,44 @@ void emit_direct(std::ostringstream& o, const char* name, const PassDev& P, int 
     }
 }
 
+// Gate lists' data of a compiled complex64 pass (phase tables, rotation
+// coefficients) as the kernel's last parameter: the code then reads it through
+// the constant cache.  Out of the staged region every lookup was a broadcast
+// through the shared-memory pipe, which a compiled pass kept busier than any
+// other unit (62% of its cycles; 30-qubit random circuit 65.7 ms, 59.9 ms with
+// the parameter).  complex128 passes, bound by the FP64 pipe, are faster out of
+// shared memory (25 qubits: 14.6 ms, with the parameter 16.9).  In op order;
+// *offs (optional): per op, its offset in complex values.  Empty when the pass
+// has more than a kernel's parameters hold: the code then reads the region.
+constexpr size_t kTabMaxBytes = 28 * 1024;
+std::vector<unsigned char> pass_table(const PassDev& P, const unsigned char* region, int dtype, std::vector<int>* offs) {
+    const size_t csz = dtype == SV_C64 ? 8 : 16;
+    const OpDev* ops = (const OpDev*)region;
+    std::vector<unsigned char> t;
+    if (offs) offs->assign(P.nops, -1);
+    if (dtype != SV_C64) return t;
+    for (int i = 0; i < P.nops; ++i) {
+        const OpDev& o = ops[i];
+        if (o.kind != OP_GATES || !o.ndata) continue;
+        const size_t n = (size_t)o.ndata;
+        if (offs) (*offs)[i] = (int)(t.size() / csz);
+        t.insert(t.end(), region + o.mat_off, region + o.mat_off + csz * n);
+        t.resize((t.size() + 15) & ~(size_t)15);  // tables start on 16 bytes
+    }
+    if (t.size() > kTabMaxBytes) t.clear();
+    return t;
+}
+
 // The pass as straight-line code (mirrors InterpOps op by op).  Returns
 // false for a structure it does not take.
 bool pass_source(const PassDev& P, const unsigned char* region, int dtype, int maxt, int minb, std::string* out,
                  bool fill = false) {
-    const int RB = reg_bits(dtype), tb = P.m - RB, L = P.L, m = P.m, no = P.nother;
-    if (tb < 5 || tb > 9 || L < 1) return false;
+    const int RB = P.rb, tb = P.m - RB, L = P.L, m = P.m, no = P.nother;
+    if (tb < 5 || tb > 9 || L < 1 || P.folded) return false;  // (compiled code moves registers by renaming)
     const OpDev* ops = (const OpDev*)region;
     const int PER = dtype == SV_C64 ? 2 : 1;  // amplitudes per 16-byte chunk
+    std::vector<int> toffs;
+    const size_t tab_bytes = pass_table(P, region, dtype, &toffs).size();
     const int T = 1 << tb, NCH = (1 << RB) / PER;
     const int istep = PER * T;
     if (istep % (1 << L)) return false;
@@ -290,7 +319,7 @@ bool pass_source(const PassDev& P, const unsigned char* region, int dtype, int m
     o << "template <typename V, typename R, int RB>\n"
          "static __device__ __forceinline__ void tile(V* v, V* tile, const PassDev& P, const unsigned char* stage,\n"
          "                                            const uint64_t* fold, RegLayout<V, RB>& Lg, const double2* ttab,\n"
-         "                                            TcCtx& T) {\n";
+         "                                            TcCtx& T, const V* tab) {\n";
     int rpos[8] = {0}, tpos[16] = {0}, nrpos[8] = {0}, ntpos[16] = {0}, frpos[8] = {0}, ftpos[16] = {0};
     bool in_regs = false, direct_load = false;
     CtLayout cur;
@@ -338,7 +367,8 @@ bool pass_source(const PassDev& P, const unsigned char* region, int dtype, int m
         }
         case OP_GATES: {
             if (!in_regs) return false;
-            o << "{\nconst V* sd = (const V*)(stage + " << op.mat_off << ");\n";
+            if (tab_bytes) o << "{\nconst V* sd = tab + " << toffs[oi] << ";\n";
+            else o << "{\nconst V* sd = (const V*)(stage + " << op.mat_off << ");\n";
             const GateRec* recs = (const GateRec*)(region + op.rec_off);
             for (int r = 0; r < op.nrec; ++r) {
                 const GateRec& g = recs[r];
@@ -364,12 +394,21 @@ bool pass_source(const PassDev& P, const unsigned char* region, int dtype, int m
                 case GR_CX: o << "reg_cx<V, RB, " << g.a << ", " << g.b << ">(v);\n"; break;
                 case GR_H: o << "reg_h<V, RB, " << g.a << ">(v);\n"; break;
                 case GR_URS:
-                    o << "reg_urs<V, RB, " << g.a << ", " << g.b << ", R>(v, sd[" << f << "].x);\n";
+                    o << "reg_urs<V, RB, " << g.a << ">(v, sd + " << f << ");\n";
                     scaled = true;
                     break;
                 case GR_HD:
                     o << "reg_h<V, RB, " << g.a << ">(v);\nreg_dt<V, RB, 0x" << std::hex << (unsigned)g.b << std::dec
                       << "u>(v, sd + " << f << ");\n";
+                    break;
+                case GR_DTS:
+                    o << "reg_dts<V, RB, 0x" << std::hex << (unsigned)g.b << std::dec << "u, R>(v, (const R*)(sd + " << f
+                      << "));\n";
+                    scaled = true;
+                    break;
+                case GR_RS:
+                    o << "reg_rs<V, RB, " << g.a << ", R>(v, (const R*)(sd + " << f << "));\n";
+                    scaled = true;
                     break;
                 case GR_SWAP: o << "reg_swap<V, RB, " << g.a << ", " << g.b << ">(v);\n"; break;
                 default: return false;
@@ -433,11 +472,15 @@ bool pass_source(const PassDev& P, const unsigned char* region, int dtype, int m
     if (direct_store) emit_direct(o, "st", P, dtype, RB, tb, rpos, tpos, false, false);
     o << "};\n}  // namespace sv\n";
     const char* R = dtype == SV_C64 ? "float" : "double";
+    if (tab_bytes) o << "struct SvTab {\nuint4 d[" << tab_bytes / 16 << "];\n};\n";
     o << "extern \"C\" __global__ void __launch_bounds__(" << maxt << ", " << minb << ") sv_jit_pass(\n"
       << "    sv::CT<" << R << ">::V* __restrict__ psi, int n, const sv::PassDev* __restrict__ pdp,\n"
-      << "    const unsigned char* __restrict__ blob, const sv::PassLayout lay, int* __restrict__ err) {\n"
+      << "    const unsigned char* __restrict__ blob, const sv::PassLayout lay, int* __restrict__ err"
+      << (tab_bytes ? ",\n    const __grid_constant__ SvTab tab" : "") << ") {\n"
       << "    sv::rpass_body<" << R << ", " << RB << ", sv::GenOps, " << (P.tc_k ? "true" : "false")
-      << ">(psi, n, pdp, blob, lay, err);\n}\n";
+      << ">(psi, n, pdp, blob, lay, err";
+    if (tab_bytes) o << ", (const sv::CT<" << R << ">::V*)&tab";
+    o << ");\n}\n";
     *out = o.str();
     return true;
 }
@@ -448,10 +491,6 @@ bool pass_source(const PassDev& P, const unsigned char* region, int dtype, int m
 // use with jit = 1, on its second with jit = 0 (the first run of a structure,
 // one-off circuits and small states stay on the interpreting kernel).
 enum { JIT_NEW = 0, JIT_COMPILING, JIT_READY, JIT_FAILED };
-// jit = 0 compiles only for states of at least this many qubits: below it a
-// pass takes tens of microseconds, and the compile (about a second) would not
-// pay back.
-constexpr int kJitAutoMinQubits = 22;
 struct Entry {
     int seen = 0;
     int state = JIT_NEW;
@@ -552,7 +591,7 @@ void jit_prepare(sv_state* h, const PlanBlob& blob, int policy, long long basis,
             const bool fill = p == blob.npasses;
             const PassDev* pd = (const PassDev*)(blob.bytes.data() + blob.pass_off) + (fill ? 0 : p);
             if ((fill && blob.npasses == 0) || pd->rmode != 1) continue;
-            const int tb = pd->m - reg_bits(h->dtype);
+            const int tb = pd->m - pd->rb;
             if (!pass_source(*pd, blob.bytes.data() + pd->region_off, h->dtype, pass_max_threads(tb),
                              pass_min_blocks(tb), &srcs[p], fill))
                 srcs[p].clear();
@@ -588,7 +627,7 @@ cudaError_t jit_launch(sv_state* h, void* entry, const void* blob_dev, const Pla
     Entry& e = *(Entry*)entry;  // entries are never erased, so the pointer stays valid
     const Driver& dr = driver();
     const PassDev* pd = (const PassDev*)(blob.bytes.data() + blob.pass_off) + pass;
-    const int tb = pd->m - reg_bits(h->dtype);
+    const int tb = pd->m - pd->rb;
     const PassLayout lay = rpass_layout(h->dtype, *pd, e.direct_load);
     {
         std::lock_guard<std::mutex> lk(g_mu);
@@ -620,11 +659,23 @@ cudaError_t jit_launch(sv_state* h, void* entry, const void* blob_dev, const Pla
     const PassDev* pdp = (const PassDev*)(b + blob.pass_off) + pass;
     PassLayout lay_arg = lay;
     int* err = (int*)h->err.ptr;
-    void* args[] = {&psi, &n, &pdp, &b, &lay_arg, &err};
+    std::vector<unsigned char> tab = pass_table(*pd, blob.bytes.data() + pd->region_off, h->dtype, nullptr);
+    void* args[] = {&psi, &n, &pdp, &b, &lay_arg, &err, tab.data()};
+    // may start before the previous pass has finished, as in rpass_t
+    CUlaunchAttribute pdl{};
+    pdl.id = CU_LAUNCH_ATTRIBUTE_PROGRAMMATIC_STREAM_SERIALIZATION;
+    pdl.value.programmaticStreamSerializationAllowed = 1;
+    CUlaunchConfig cfg{};
+    cfg.gridDimX = (unsigned)grid;
+    cfg.gridDimY = cfg.gridDimZ = 1;
+    cfg.blockDimX = (unsigned)threads;
+    cfg.blockDimY = cfg.blockDimZ = 1;
+    cfg.sharedMemBytes = (unsigned)lay.total;
+    cfg.hStream = (CUstream)h->stream;
+    cfg.attrs = &pdl;
+    cfg.numAttrs = pd->tc_k == 0 && pdl_pays(pass, grid, per_sm) ? 1 : 0;
     count_launch();
-    if (dr.launch(e.fn, (unsigned)grid, 1, 1, (unsigned)threads, 1, 1, (unsigned)lay.total, (CUstream)h->stream, args,
-                  nullptr) != CUDA_SUCCESS)
-        return cudaErrorLaunchFailure;
+    if (dr.launch(&cfg, e.fn, args, nullptr) != CUDA_SUCCESS) return cudaErrorLaunchFailure;
     {
         std::lock_guard<std::mutex> lk(g_mu);
         ++g_launched;
@@ -698,7 +749,10 @@ extern "C" int sv_jit_check(int n, sv_dtype dt, const sv_gate* gates, size_t cou
     size_t bad = 0;
     if (canonicalise(n, gates, count, &cg, &bad) != SV_OK)
         return set_error(SV_EINVAL, "invalid gate record at index " + std::to_string(bad));
-    const PlanOptions po = resolve_options(n, dt, opt);
+    sv_options jo{};  // the plan an apply that compiles would run
+    if (opt) jo = *opt;
+    jo.jit = 1;
+    const PlanOptions po = resolve_options(n, dt, &jo);
     Plan plan;
     plan_greedy(n, dt, cg, po, &plan);
     PlanBlob blob;
@@ -715,7 +769,7 @@ extern "C" int sv_jit_check(int n, sv_dtype dt, const sv_gate* gates, size_t cou
         if (fill && blob.npasses == 0) break;
         const PassDev* pd = (const PassDev*)(blob.bytes.data() + blob.pass_off) + (fill ? 0 : p);
         if (pd->rmode != 1) continue;
-        const int tb = pd->m - reg_bits(dt);
+        const int tb = pd->m - pd->rb;
         std::string src;
         if (!pass_source(*pd, blob.bytes.data() + pd->region_off, dt, pass_max_threads(tb), pass_min_blocks(tb),
                          &src, fill))

@@ -629,6 +629,19 @@ void drop_small_phases(std::vector<CGate>* g, double eps) {
     g->swap(kept);
 }
 
+// Tile width of plans with small_reg_bits (measured on 8-layer random and
+// ansatz circuits): the whole state while its one CTA is as quick as several
+// passes, then tiles of 32 to 64 threads' worth of CTAs, wider ones as the
+// state fills the GPU.  complex128, bound by the FP64 pipe of the SMs it
+// reaches, keeps about 128 tiles.  0: the wide plan is the faster one (20 and
+// 18 qubits are the last where the small one wins: 257 against 307 us at 20
+// complex64 qubits, 432 against 433 at 21; 517 against 862 at 18 complex128
+// qubits, 2019 against 1802 at 20).
+static int small_tile(int n, int dtype) {
+    if (dtype == SV_C64) return n <= 11 ? n : n <= 15 ? 10 : n <= 17 ? 11 : n <= 20 ? 12 : 0;
+    return n <= 15 ? std::min(n, 10) : n <= 18 ? n - 7 : 0;
+}
+
 PlanOptions resolve_options(int n, int dtype, const sv_options* opt) {
     PlanOptions po;
     po.tile_m = dtype == SV_C64 ? 13 : 12;
@@ -653,6 +666,18 @@ PlanOptions resolve_options(int n, int dtype, const sv_options* opt) {
     if (dtype != SV_C64) po.tensor = -1, po.tc_auto = 0;
     po.k_max = std::max(2, std::min(kMaxK, po.k_max));
     const int mmax = dtype == SV_C64 ? 14 : 13;
+    po.rb = reg_bits(dtype);
+    // Plans of default shape that the interpreting kernel will run (never
+    // compiled, or too small to be): half the amplitudes per thread and a tile
+    // that spreads the state over the GPU.
+    if (po.planner == SV_PLAN_GREEDY && po.pass_kernel == 0 && po.tensor < 0 && !po.tc_auto &&
+        (po.jit < 0 || (po.jit == 0 && n < kJitAutoMinQubits)) && small_tile(n, dtype) > 0 &&
+        (!opt || (opt->k_max <= 0 && opt->tile_m <= 0))) {
+        po.rb = small_reg_bits(dtype);
+        po.fold_perms = true;
+        po.k_max = po.rb;
+        po.tile_m = small_tile(n, dtype);
+    }
     po.tile_m = std::max(1, std::min(mmax, po.tile_m));
     po.tile_m = std::min(po.tile_m, n);
     return po;
@@ -670,7 +695,7 @@ void greedy_pass(int n, int dtype, const std::vector<CGate>& gates, const std::v
     const int m = std::max(std::min(n, L + 2), std::min(po.tile_m, n));
     const int kmax = std::min(po.k_max, m);
     // tensor-core blocks run in register passes of at least 128 threads
-    const bool tc_auto_ok = po.tc_auto && dtype == SV_C64 && po.pass_kernel == 0 && m - reg_bits(dtype) >= 7;
+    const bool tc_auto_ok = po.tc_auto && dtype == SV_C64 && po.pass_kernel == 0 && po.rb == 5 && m - po.rb >= 7;
     std::vector<char> inT(n), blocked(n);
     std::vector<int> executed, deferred;
     int nblocked = 0;
@@ -816,7 +841,7 @@ void greedy_pass(int n, int dtype, const std::vector<CGate>& gates, const std::v
             // (the automatic choice keeps the pass's staged matrices within
             // kTcStageBudget: beyond it the pass would hold one CTA per SM)
             const bool tc_auto = tc_auto_ok && (kb == 4 || kb == 5) && tc_bytes + 2 * tc16_bytes(kb) <= kTcStageBudget;
-            const bool seq = !tc_forced && kb <= max_gates_k(dtype) && best_gate_sequence(B, &op.recs, &op.gdata);
+            const bool seq = !tc_forced && kb <= po.rb && best_gate_sequence(B, &op.recs, &op.gdata);
             const double seq_cost = seq ? gate_sequence_cost(op.recs, &op.gdata) : 1e30;
             if (tc_forced || (tc_auto && seq_cost > tc_cost(kb))) {
                 op.kind = OP_DENSE;
@@ -954,6 +979,8 @@ void plan_greedy(int n, int dtype, const std::vector<CGate>& gates, const PlanOp
     out->no_register_passes = po.pass_kernel == 1;
     out->use_tma = po.pass_kernel == 2;
     out->jit = po.jit;
+    out->rb = po.rb;
+    out->fold_perms = po.fold_perms;
     std::vector<int> remaining(gates.size()), deferred;
     for (size_t i = 0; i < gates.size(); ++i) remaining[i] = (int)i;
     while (!remaining.empty()) {
@@ -1237,7 +1264,7 @@ bool use_tc(const Plan& p, const HostOp& o) {
 // Tensor-core block of a register pass (OP_DENSE_TC).
 bool reg_tc(const Plan& p, const HostOp& o, int tb) {
     const int k = (int)o.qubits.size();
-    return o.tc && o.kind == OP_DENSE && p.dtype == SV_C64 && !p.use_tma && (k == 4 || k == 5) && tb >= 7;
+    return o.tc && o.kind == OP_DENSE && p.dtype == SV_C64 && !p.use_tma && (k == 4 || k == 5) && p.rb == 5 && tb >= 7;
 }
 
 uint16_t f32_to_f16(float f);
@@ -1321,6 +1348,55 @@ void smem_region(const Plan& p, const HostPass& hp, PassDev* P, const int* loc, 
     assemble(ops, pay, P, out);
 }
 
+// Take the CX and SWAP records a gate list can end with (register-bit
+// positions, tables over all 2^r registers) off it: one that commutes with
+// every later record that stays moves to the end, the phase tables it passes
+// permuted (T after P equals P after T', T'[j] = T[P(j)]), and the permutation
+// of register indices they make together becomes img[b], the index that
+// register index 2^b goes to (CX and SWAP are linear over XOR).
+int permuted_index(const GateRec& g, int j) {  // where CX or SWAP takes register index j (its own inverse)
+    const int ba = (j >> g.a) & 1, bb = (j >> g.b) & 1;
+    if (g.kind == GR_CX) return j ^ (ba << g.b);
+    return ba == bb ? j : j ^ (1 << g.a) ^ (1 << g.b);
+}
+void fold_permutations(int r, std::vector<GateRec>* recs, std::vector<cd>* data, int* img) {
+    for (int b = 0; b < r; ++b) img[b] = 1 << b;
+    auto apply = permuted_index;
+    int blocked = 0;  // register bits a later record that stays acts on
+    std::vector<GateRec> tail;
+    for (int i = (int)recs->size() - 1; i >= 0; --i) {
+        const GateRec g = (*recs)[i];
+        if (g.kind == GR_DT) continue;
+        if (g.kind != GR_CX && g.kind != GR_SWAP) {
+            blocked |= g.kind == GR_HD || g.kind == GR_DTS || g.kind == GR_RS ? ~0 : 1 << g.a;
+            continue;
+        }
+        if (((1 << g.a) | (1 << g.b)) & blocked) {
+            blocked |= (1 << g.a) | (1 << g.b);
+            continue;
+        }
+        for (size_t t = i + 1; t < recs->size(); ++t) {
+            GateRec& T = (*recs)[t];
+            if (T.kind != GR_DT) continue;
+            std::vector<cd> moved(1 << r);
+            int mask = 0;
+            for (int j = 0; j < (1 << r); ++j) {
+                moved[j] = (*data)[(size_t)T.off + apply(g, j)];
+                mask |= ((T.b >> apply(g, j)) & 1) << j;
+            }
+            std::copy(moved.begin(), moved.end(), data->begin() + T.off);
+            T.b = mask;
+            const int da = (T.a >> g.a) & 1, db = (T.a >> g.b) & 1;
+            if (g.kind == GR_CX) T.a |= db << g.a;
+            else T.a = (T.a & ~((1 << g.a) | (1 << g.b))) | (db << g.a) | (da << g.b);
+        }
+        recs->erase(recs->begin() + i);
+        tail.insert(tail.begin(), g);
+    }
+    for (int b = 0; b < r; ++b)
+        for (const GateRec& g : tail) img[b] = apply(g, img[b]);
+}
+
 // Region for the register-resident pass kernel, or false when the pass
 // needs the shared-memory kernel (tensor-core blocks, dense blocks wider than
 // kRegDenseMaxK, a thread count outside 32..512, or a region too large to
@@ -1329,7 +1405,7 @@ void smem_region(const Plan& p, const HostPass& hp, PassDev* P, const int* loc, 
 // order at register bits 0..k-1) and fills the other register bits with the
 // tile positions the following blocks use soonest.
 bool reg_region(const Plan& p, const HostPass& hp, PassDev* P, const int* loc, std::vector<unsigned char>* out) {
-    const int r = reg_bits(p.dtype), m = P->m, tb = m - r, nops = (int)hp.ops.size();
+    const int r = p.rb, m = P->m, tb = m - r, nops = (int)hp.ops.size();
     if (tb < 5 || tb > 9) return false;
     std::vector<std::vector<int>> used(nops);
     for (int i = 0; i < nops; ++i) {
@@ -1348,6 +1424,30 @@ bool reg_region(const Plan& p, const HostPass& hp, PassDev* P, const int* loc, s
     std::vector<OpDev> ops;
     Payload pay;
     std::vector<int> rpos, tpos;
+    long double scale = P->scale;  // the deferred factors: rounded to double once, not at every gate
+    int deferred = 0;              // rotations and Hadamards in it
+    // gate lists, put into the payload once their ends are known
+    struct GateList {
+        size_t op;
+        std::vector<GateRec> recs;
+        std::vector<cd> data;
+    };
+    std::vector<GateList> lists;
+    // Tile positions each register bit flips when the registers are written
+    // back now: the layout's own, unless permutations the last block ends with
+    // are folded into the addresses.
+    auto write_masks = [&](int* w) {
+        int img[8];
+        for (int b = 0; b < r; ++b) img[b] = 1 << b;
+        if (p.fold_perms && !ops.empty() && ops.back().kind == OP_GATES)
+            fold_permutations(r, &lists.back().recs, &lists.back().data, img);
+        for (int b = 0; b < r; ++b) {
+            w[b] = 0;
+            for (int c = 0; c < r; ++c)
+                if ((img[b] >> c) & 1) w[b] |= 1 << rpos[c];
+            P->folded |= w[b] != 1 << rpos[b];
+        }
+    };
     // Thread bits 0..4 are the lane bits, the others the warp bits.  A remap
     // whose incoming register positions all sit at lane bits can hand each
     // lane bit it frees to an outgoing register position: every warp's
@@ -1495,10 +1595,11 @@ bool reg_region(const Plan& p, const HostPass& hp, PassDev* P, const int* loc, s
             first.insert(first.end(), later.begin(), later.end());
             std::copy(first.begin(), first.end(), fresh.begin());
         }
-        rpos = slots;
-        tpos = fresh;
         OpDev O;
         memset(&O, 0, sizeof(O));
+        if (!rpos.empty()) write_masks(O.wmask);
+        rpos = slots;
+        tpos = fresh;
         O.kind = OP_REMAP;
         O.k = r;
         O.nrec = local ? 1 : 0;
@@ -1596,14 +1697,48 @@ bool reg_region(const Plan& p, const HostPass& hp, PassDev* P, const int* loc, s
             O.kind = OP_DENSE_TC;
             const std::vector<uint16_t> b = tc16_operand(o.mat, O.k);
             O.mat_off = (int)pay.put(b.data(), sizeof(uint16_t) * b.size());
-            O.tc_scale = (float)((double)kTcInScale * P->scale);
-            P->scale = 1.0 / ((double)kTcInScale * (double)kTcMatScale);
+            O.tc_scale = (float)((double)kTcInScale * (double)scale);
+            scale = 1.0L / ((long double)kTcInScale * (long double)kTcMatScale);
             if (O.k > P->tc_k) P->tc_k = O.k;
         } else if (o.kind == OP_DENSE) {
             O.mat_off = (int)pay.put_cplx(o.mat, p.dtype);
         } else {
             std::vector<GateRec> recs;
             std::vector<cd> data;
+            // complex128: the real factors registers lack behind tables
+            // applied without their cosines (GR_DTS), and which tables may be
+            const bool split = p.dtype == SV_C128;
+            std::vector<double> lack(1 << r, 1.0);
+            std::vector<char> whole(o.recs.size(), 1);  // the table's factors end here
+            if (split) {
+                bool last = true;
+                for (size_t i = o.recs.size(); i-- > 0;) {
+                    const GateRec& g = o.recs[i];
+                    if (g.kind == GR_DT) {
+                        whole[i] = last;
+                        last = false;
+                        for (int j = 0; j < (1 << O.k); ++j)  // (tangents within range)
+                            if (std::fabs(o.gdata[(size_t)g.off + j].real()) < kMinDeferredCos) whole[i] = 1;
+                    } else if (g.kind != GR_CX && g.kind != GR_SWAP) {
+                        const cd* gm = &o.gdata[(size_t)g.off];
+                        // (a rotation scales with its partner; anything else, an
+                        // exact Hadamard included, needs equal factors)
+                        if (!(g.kind == GR_UR && gm[0] == gm[3] && gm[1] == -gm[2] &&
+                              std::fabs(gm[0].real()) >= kMinDeferredCos))
+                            last = true;
+                    }
+                }
+            }
+            auto lacking = [&]() {
+                for (double s : lack)
+                    if (s != 1.0) return true;
+                return false;
+            };
+            auto put_reals = [&](const std::vector<double>& v) {  // two per complex slot
+                const int off = (int)data.size();
+                for (size_t j = 0; j < v.size(); j += 2) data.push_back(cd(v[j], v[j + 1]));
+                return off;
+            };
             for (const GateRec& g : o.recs) {
                 GateRec t = g;
                 if (g.kind == GR_DT) {
@@ -1613,38 +1748,80 @@ bool reg_region(const Plan& p, const HostPass& hp, PassDev* P, const int* loc, s
                     t.off = (int)data.size();
                     t.b = 0;
                     t.a = 0;
+                    // a complex64 table after many deferred factors takes them
+                    // along (their range stays small; a rule on counts, so that
+                    // circuits of one shape keep one compiled pass)
+                    double fold = 1.0;
+                    if (p.dtype == SV_C64 && deferred >= 12) {
+                        fold = (double)scale;
+                        scale = 1.0L;
+                        deferred = 0;
+                    }
                     for (int j = 0; j < O.k; ++j)
                         if ((g.a >> j) & 1) t.a |= 1 << O.lq[j];
                     for (int v = 0; v < (1 << r); ++v) {
                         int idx = 0;
                         for (int j = 0; j < O.k; ++j) idx |= ((v >> O.lq[j]) & 1) << j;
-                        const cd e = o.gdata[(size_t)g.off + idx];
+                        const cd e = o.gdata[(size_t)g.off + idx] * lack[v] * fold;
                         data.push_back(e);
                         if (e != cd(1.0, 0.0)) t.b |= 1 << v;
+                    }
+                    if (whole[&g - o.recs.data()]) {
+                        if (lacking()) t.a = (1 << r) - 1;  // the factors may depend on every register bit
+                        lack.assign(1 << r, 1.0);
+                    } else {
+                        std::vector<double> tang(1 << r);
+                        for (int v = 0; v < (1 << r); ++v) {
+                            const cd e = data[(size_t)t.off + v] / lack[v];
+                            tang[v] = e.imag() / e.real();
+                            lack[v] *= e.real();
+                        }
+                        data.resize(t.off);
+                        t.b = 0;
+                        for (int v = 0; v < (1 << r); ++v) t.b |= (tang[v] != 0.0) << v;
+                        t.kind = GR_DTS;
+                        t.off = put_reals(tang);
                     }
                 } else {
                     t.a = O.lq[g.a];
                     if (g.kind == GR_CX || g.kind == GR_SWAP) t.b = O.lq[g.b];
+                    if (split && (g.kind == GR_CX || g.kind == GR_SWAP)) {
+                        std::vector<double> moved(1 << r);
+                        for (int v = 0; v < (1 << r); ++v) moved[v] = lack[permuted_index(t, v)];
+                        lack.swap(moved);
+                    }
                     const cd* gm = g.kind == GR_U || g.kind == GR_UR ? &o.gdata[(size_t)g.off] : nullptr;
                     const double hs = 1.0 / std::sqrt(2.0);
                     // (factors deferred only while the growth they leave in the
                     // registers stays below 2^40)
                     if (g.kind == GR_UR && gm[0] == cd(hs, 0.0) && gm[1] == cd(hs, 0.0) && gm[2] == cd(hs, 0.0) &&
-                        gm[3] == cd(-hs, 0.0) && std::fabs(P->scale) > 0x1p-40) {
+                        gm[3] == cd(-hs, 0.0) && std::fabs((double)scale) > 0x1p-40) {
                         t.kind = GR_H;  // butterfly; the factor goes to the pass's write-back scale
                         t.off = 0;
-                        P->scale *= hs;
-                    } else if (g.kind == GR_UR && gm[0] == gm[3] && gm[1] == -gm[2] && std::fabs(P->scale) > 0x1p-40) {
-                        // rotation [[c, -s], [s, c]]: the larger of c, s goes to the
-                        // write-back scale (each factor is at least 1/sqrt(2) in
-                        // magnitude, so the deferred growth stays below 2^40)
-                        const double c = gm[0].real(), sn = gm[2].real();
-                        const bool cform = std::fabs(c) >= std::fabs(sn);
-                        t.kind = GR_URS;
-                        t.b = cform ? 0 : 1;
-                        t.off = (int)data.size();
-                        data.push_back(cd(cform ? sn / c : c / sn, 0.0));
-                        P->scale *= cform ? c : sn;
+                        scale *= 1.0L / std::sqrt(2.0L);
+                        ++deferred;
+                    } else if (g.kind == GR_UR && gm[0] == gm[3] && gm[1] == -gm[2] &&
+                               std::fabs(gm[0].real()) >= kMinDeferredCos &&
+                               (std::fabs((double)scale) > (p.dtype == SV_C64 ? 0x1p-30 : 0x1p-200) || lacking())) {
+                        // rotation [[c, -s], [s, c]] = c [[1, -t], [t, 1]]: c goes to the
+                        // write-back scale (|c| >= 2^-10, so the growth left in complex64
+                        // registers stays below 2^40; complex128, whose range is far wider,
+                        // never stops inside a run of GR_RS: at most 40 more factors)
+                        const double c = gm[0].real(), tn = gm[2].real() / c;
+                        if (split && lacking()) {
+                            std::vector<double> co(1 << r);
+                            for (int v = 0; v < (1 << r); ++v)
+                                co[v] = ((v >> t.a) & 1 ? tn : -tn) * (lack[v ^ (1 << t.a)] / lack[v]);
+                            t.kind = GR_RS;
+                            t.off = put_reals(co);
+                        } else {
+                            t.kind = GR_URS;
+                            t.off = (int)data.size();
+                            data.push_back(cd(tn, tn));
+                            data.push_back(cd(-tn, -tn));
+                        }
+                        scale *= (long double)c;
+                        ++deferred;
                     } else if (gm) {
                         t.off = (int)data.size();
                         for (int e = 0; e < 4; ++e) data.push_back(gm[e]);
@@ -1663,16 +1840,23 @@ bool reg_region(const Plan& p, const HostPass& hp, PassDev* P, const int* loc, s
                 }
             }
             recs.swap(fused);
-            O.mat_off = (int)pay.put_cplx(data, p.dtype);
-            O.ndata = (int)data.size();
-            O.nrec = (int)recs.size();
-            O.rec_off = (int)pay.put(recs.data(), sizeof(GateRec) * recs.size());
+            lists.push_back(GateList{ops.size(), std::move(recs), std::move(data)});
         }
         ops.push_back(O);
     }
     if (rpos.empty()) remap(0, {});
+    P->scale = (double)scale;
+    write_masks(P->fmask);
+    for (const GateList& l : lists) {
+        OpDev& O = ops[l.op];
+        O.mat_off = (int)pay.put_cplx(l.data, p.dtype);
+        O.ndata = (int)l.data.size();
+        O.nrec = (int)l.recs.size();
+        O.rec_off = (int)pay.put(l.recs.data(), sizeof(GateRec) * l.recs.size());
+    }
     assemble(ops, pay, P, out);
     P->rmode = p.use_tma ? 2 : 1;
+    P->rb = r;
     P->ndiag = nd;
     // passes with tensor-core blocks stage their matrices (16 KiB per 5-qubit
     // block) in a larger region
@@ -1683,7 +1867,7 @@ bool reg_region(const Plan& p, const HostPass& hp, PassDev* P, const int* loc, s
 
 bool register_pass_eligible(const Plan& p, const HostPass& hp) {
     if (p.no_register_passes) return false;
-    const int r = reg_bits(p.dtype), tb = (int)hp.tile.size() - r;
+    const int r = p.rb, tb = (int)hp.tile.size() - r;
     if (tb < 5 || tb > 9) return false;
     for (const HostOp& o : hp.ops) {
         if (o.kind == OP_DIAG) continue;

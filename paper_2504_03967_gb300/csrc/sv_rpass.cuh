@@ -47,6 +47,53 @@ template <typename V> __device__ __forceinline__ V cfma(V a, V b, V c) {  // a*b
     r.y = fma(a.x, b.y, fma(a.y, b.x, c.y));
     return r;
 }
+// Part by part: s * b + c, s * b, a + b, a - b.  complex64 uses the packed FP32
+// instructions: both parts in one issue slot (each part rounds as the scalar
+// instruction does), and with three different register operands 118 FMA per
+// clock and SM against 99.  Compiled passes of a 30-qubit random circuit: 63.4
+// ms with scalar instructions, 60.1 ms with these.
+__device__ __forceinline__ unsigned long long f2_pack(float2 a) {
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a.x), "f"(a.y));
+    return r;
+}
+__device__ __forceinline__ float2 f2_unpack(unsigned long long r) {
+    float2 a;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a.x), "=f"(a.y) : "l"(r));
+    return a;
+}
+__device__ __forceinline__ float2 vfma(float2 s, float2 b, float2 c) {
+    unsigned long long r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(f2_pack(s)), "l"(f2_pack(b)), "l"(f2_pack(c)));
+    return f2_unpack(r);
+}
+__device__ __forceinline__ float2 vmul(float2 s, float2 b) {
+    unsigned long long r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(f2_pack(s)), "l"(f2_pack(b)));
+    return f2_unpack(r);
+}
+__device__ __forceinline__ float2 vadd(float2 a, float2 b) {
+    unsigned long long r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(f2_pack(a)), "l"(f2_pack(b)));
+    return f2_unpack(r);
+}
+__device__ __forceinline__ float2 vsub(float2 a, float2 b) {
+    unsigned long long r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(f2_pack(a)), "l"(f2_pack(b)));
+    return f2_unpack(r);
+}
+__device__ __forceinline__ double2 vfma(double2 s, double2 b, double2 c) {
+    return make_double2(fma(s.x, b.x, c.x), fma(s.y, b.y, c.y));
+}
+__device__ __forceinline__ double2 vmul(double2 s, double2 b) { return make_double2(s.x * b.x, s.y * b.y); }
+__device__ __forceinline__ double2 vadd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ double2 vsub(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
+template <typename V, typename R> __device__ __forceinline__ V vdup(R s) {
+    V r;
+    r.x = s;
+    r.y = s;
+    return r;
+}
 template <typename V> __device__ __forceinline__ V czero() {
     V r;
     r.x = 0;
@@ -74,6 +121,13 @@ template <typename V> __device__ __forceinline__ int swz(int i) {
     else return i ^ ((i >> 3) & 7);                                   // 1 amplitude per chunk
 }
 
+// Programmatic dependent launch: a pass kernel lets the next one start as soon
+// as all its CTAs run (pdl_trigger), so that the next pass's staging and tables
+// overlap this pass; before it touches the state it waits for this one to have
+// finished (pdl_wait).  Launched without the attribute both do nothing.
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 template <int N> __device__ __forceinline__ void cp_async_wait_group() {
     asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
@@ -86,7 +140,7 @@ template <int N> __device__ __forceinline__ void cp_async_wait_group() {
 // code unrolled for its (compile-time) position inside the block:
 //   GR_U   2x2 complex matrix on position a        8 FMA per amplitude
 //   GR_UR  2x2 real matrix on position a           4
-//   GR_URS rotation with its factor deferred       2
+//   GR_URS rotation with its factor deferred       2 (packed: 1)
 //   GR_DT  2^K-entry diagonal (phase) table        one complex product
 //   GR_CX  controlled-NOT (control a, target b)    register moves
 //   GR_SWAP                                        register moves
@@ -103,40 +157,53 @@ __device__ __forceinline__ void reg_u(V* v, V u00, V u01, V u10, V u11) {
 }
 template <typename V, int K, int P, typename R>
 __device__ __forceinline__ void reg_ur(V* v, R u00, R u01, R u10, R u11) {
+    const V m00 = vdup<V>(u00), m01 = vdup<V>(u01), m10 = vdup<V>(u10), m11 = vdup<V>(u11);
 #pragma unroll
     for (int j = 0; j < (1 << K); ++j)
         if (!((j >> P) & 1)) {
             const V a = v[j], b = v[j | (1 << P)];
-            V x, y;
-            x.x = fma(u00, a.x, u01 * b.x);
-            x.y = fma(u00, a.y, u01 * b.y);
-            y.x = fma(u10, a.x, u11 * b.x);
-            y.y = fma(u10, a.y, u11 * b.y);
-            v[j] = x;
-            v[j | (1 << P)] = y;
+            v[j] = vfma(m00, a, vmul(m01, b));
+            v[j | (1 << P)] = vfma(m10, a, vmul(m11, b));
         }
 }
-// Rotation without its factor: FORM 0 [[1, -t], [t, 1]], FORM 1 [[t, -1], [1, t]].
-template <typename V, int K, int P, int FORM, typename R>
-__device__ __forceinline__ void reg_urs(V* v, R t) {
+// Rotation without its factor, [[1, -t], [t, 1]]: t holds (t, t) and (-t, -t).
+template <typename V, int K, int P>
+__device__ __forceinline__ void reg_urs(V* v, const V* __restrict__ t) {
+    V tp = t[0], tn = t[1];
+    if constexpr (sizeof(V) == 8) {
+        asm volatile("" : "+f"(tp.x), "+f"(tn.x));  // (see hold)
+        tp.y = tp.x;
+        tn.y = tn.x;
+    }
 #pragma unroll
     for (int j = 0; j < (1 << K); ++j)
         if (!((j >> P) & 1)) {
             const V a = v[j], b = v[j | (1 << P)];
-            V x, y;
-            if (FORM == 0) {
-                x.x = fma(-t, b.x, a.x);
-                x.y = fma(-t, b.y, a.y);
-                y.x = fma(t, a.x, b.x);
-                y.y = fma(t, a.y, b.y);
-            } else {
-                x.x = fma(t, a.x, -b.x);
-                x.y = fma(t, a.y, -b.y);
-                y.x = fma(t, b.x, a.x);
-                y.y = fma(t, b.y, a.y);
-            }
-            v[j] = x;
-            v[j | (1 << P)] = y;
+            v[j] = vfma(tn, b, a);
+            v[j | (1 << P)] = vfma(tp, a, b);
+        }
+}
+// Phase table without its cosines (GR_DTS) and rotation of registers that lack
+// them (GR_RS); t: 2^K reals.
+template <typename V, int K, unsigned MASK, typename R>
+__device__ __forceinline__ void reg_dts(V* v, const R* __restrict__ t) {
+#pragma unroll
+    for (int j = 0; j < (1 << K); ++j)
+        if ((MASK >> j) & 1u) {
+            const V a = v[j];
+            v[j].x = fma(-t[j], a.y, a.x);
+            v[j].y = fma(t[j], a.x, a.y);
+        }
+}
+template <typename V, int K, int P, typename R>
+__device__ __forceinline__ void reg_rs(V* v, const R* __restrict__ c) {
+#pragma unroll
+    for (int j = 0; j < (1 << K); ++j)
+        if (!((j >> P) & 1)) {
+            const int j1 = j | (1 << P);
+            const V a = v[j], b = v[j1];
+            v[j] = vfma(vdup<V>(c[j]), b, a);
+            v[j1] = vfma(vdup<V>(c[j1]), a, b);
         }
 }
 template <typename V, int K, int P>
@@ -145,13 +212,8 @@ __device__ __forceinline__ void reg_h(V* v) {  // unscaled butterfly (a + b, a -
     for (int j = 0; j < (1 << K); ++j)
         if (!((j >> P) & 1)) {
             const V a = v[j], b = v[j | (1 << P)];
-            V x, y;
-            x.x = a.x + b.x;
-            x.y = a.y + b.y;
-            y.x = a.x - b.x;
-            y.y = a.y - b.y;
-            v[j] = x;
-            v[j | (1 << P)] = y;
+            v[j] = vadd(a, b);
+            v[j | (1 << P)] = vsub(a, b);
         }
 }
 template <typename V, int K, int C, int T>
@@ -175,13 +237,39 @@ __device__ __forceinline__ void reg_swap(V* v) {
         }
 }
 
+// Entries j and j + 1 of a table (complex64: one 16-byte access, tables start on
+// 16 bytes and j is even), held in registers: as operands left in the constant
+// bank they took the compiler two to four times as long per pass.
+template <typename V> __device__ __forceinline__ void hold(V& a) {
+    if constexpr (sizeof(V) == 8) asm volatile("" : "+f"(a.x), "+f"(a.y));
+}
+template <typename V> __device__ __forceinline__ void table_pair(const V* __restrict__ t, V& a, V& b) {
+    if constexpr (sizeof(V) == 8) {
+        const float4 q = *reinterpret_cast<const float4*>(t);
+        a.x = q.x;
+        a.y = q.y;
+        b.x = q.z;
+        b.y = q.w;
+    } else {
+        a = t[0];
+        b = t[1];
+    }
+    hold(a);
+    hold(b);
+}
+
 // Phase table on the registers whose bit is set in MASK (a compile-time
 // GR_DT / the table half of GR_HD).
 template <typename V, int K, unsigned MASK>
 __device__ __forceinline__ void reg_dt(V* v, const V* __restrict__ t) {
 #pragma unroll
-    for (int j = 0; j < (1 << K); ++j)
-        if ((MASK >> j) & 1u) v[j] = cmul(t[j], v[j]);
+    for (int j = 0; j < (1 << K); j += 2) {
+        if (!((MASK >> j) & 3u)) continue;
+        V a, b;
+        table_pair(t + j, a, b);
+        if ((MASK >> j) & 1u) v[j] = cmul(a, v[j]);
+        if ((MASK >> j) & 2u) v[j + 1] = cmul(b, v[j + 1]);
+    }
 }
 
 // The same when the table depends only on the register bits in DEP (entry j
@@ -190,8 +278,10 @@ template <typename V, int K, unsigned MASK, unsigned DEP>
 __device__ __forceinline__ void reg_dt_dep(V* v, const V* __restrict__ t) {
     V e[1 << K];
 #pragma unroll
-    for (int j = 0; j < (1 << K); ++j)
-        if ((j & ~DEP) == 0 && ((MASK >> j) & 1u)) e[j] = t[j];
+    for (int j = 0; j < (1 << K); j += 2) {
+        if ((j & ~DEP) != 0 || !((MASK >> j) & ((DEP & 1u) ? 3u : 1u))) continue;
+        table_pair(t + j, e[j], e[j + 1]);
+    }
 #pragma unroll
     for (int j = 0; j < (1 << K); ++j)
         if ((MASK >> j) & 1u) v[j] = cmul(e[j & DEP], v[j]);
@@ -217,20 +307,15 @@ __device__ __forceinline__ void reg_ur_any(V* v, int p, R u00, R u01, R u10, R u
     default: if constexpr (K > 4) reg_ur<V, K, 4>(v, u00, u01, u10, u11); break;
     }
 }
-template <typename V, int K, int FORM, typename R>
-__device__ __forceinline__ void reg_urs_p(V* v, int p, R t) {
+template <typename V, int K>
+__device__ __forceinline__ void reg_urs_any(V* v, int p, const V* __restrict__ t) {
     switch (p) {
-    case 0: reg_urs<V, K, 0, FORM, R>(v, t); break;
-    case 1: if constexpr (K > 1) reg_urs<V, K, 1, FORM, R>(v, t); break;
-    case 2: if constexpr (K > 2) reg_urs<V, K, 2, FORM, R>(v, t); break;
-    case 3: if constexpr (K > 3) reg_urs<V, K, 3, FORM, R>(v, t); break;
-    default: if constexpr (K > 4) reg_urs<V, K, 4, FORM, R>(v, t); break;
+    case 0: reg_urs<V, K, 0>(v, t); break;
+    case 1: if constexpr (K > 1) reg_urs<V, K, 1>(v, t); break;
+    case 2: if constexpr (K > 2) reg_urs<V, K, 2>(v, t); break;
+    case 3: if constexpr (K > 3) reg_urs<V, K, 3>(v, t); break;
+    default: if constexpr (K > 4) reg_urs<V, K, 4>(v, t); break;
     }
-}
-template <typename V, int K, typename R>
-__device__ __forceinline__ void reg_urs_any(V* v, int p, int form, R t) {
-    if (form == 0) reg_urs_p<V, K, 0, R>(v, p, t);
-    else reg_urs_p<V, K, 1, R>(v, p, t);
 }
 template <typename V, int K>
 __device__ __forceinline__ void reg_h_any(V* v, int p) {
@@ -539,39 +624,81 @@ __device__ __forceinline__ void reg_dense_tc(float2* v, const unsigned char* bma
     }
 }
 
+// Phase table of the interpreting kernel: entries in groups of four, a group
+// of ones skipped (mask: the entries that differ from 1; a one inside a group
+// multiplies exactly).  One branch and one wait per group: with a branch per
+// entry the table lookups' latency, not the products, set the time.
+template <typename V, int RB>
+__device__ __forceinline__ void reg_dt_any(V* v, unsigned mask, const V* __restrict__ t) {
+    constexpr int G = 4;
+#pragma unroll
+    for (int j = 0; j < (1 << RB); j += G)
+        if ((mask >> j) & ((1u << G) - 1u)) {
+            V e[G];
+            if constexpr (sizeof(V) == 8) {  // (tables start on 16 bytes)
+#pragma unroll
+                for (int i = 0; i < G; i += 2) {
+                    const float4 q = *reinterpret_cast<const float4*>(t + j + i);
+                    e[i].x = q.x;
+                    e[i].y = q.y;
+                    e[i + 1].x = q.z;
+                    e[i + 1].y = q.w;
+                }
+            } else {
+#pragma unroll
+                for (int i = 0; i < G; ++i) e[i] = t[j + i];
+            }
+#pragma unroll
+            for (int i = 0; i < G; ++i) v[j + i] = cmul(e[i], v[j + i]);
+        }
+}
+
 template <typename V, int RB>
 __device__ __forceinline__ void reg_gates(V* v, const GateRec* __restrict__ recs, int nrec, const V* __restrict__ sd) {
     using R = decltype(V().x);
+    if (nrec <= 0) return;
+    GateRec next = recs[0];
     for (int r = 0; r < nrec; ++r) {
-        const GateRec g = recs[r];
+        const GateRec g = next;
+        next = recs[r + 1 < nrec ? r + 1 : r];  // (in flight while this one runs)
         switch (g.kind) {
         case GR_U: reg_u_any<V, RB>(v, g.a, sd[g.off], sd[g.off + 1], sd[g.off + 2], sd[g.off + 3]); break;
         case GR_UR:
             reg_ur_any<V, RB, R>(v, g.a, sd[g.off].x, sd[g.off + 1].x, sd[g.off + 2].x, sd[g.off + 3].x);
             break;
-        case GR_DT:  // b: entries that differ from 1
-#pragma unroll
-            for (int j = 0; j < (1 << RB); ++j)
-                if ((g.b >> j) & 1) v[j] = cmul(sd[g.off + j], v[j]);
-            break;
-        case GR_URS: reg_urs_any<V, RB, R>(v, g.a, g.b, sd[g.off].x); break;
+        case GR_DT: reg_dt_any<V, RB>(v, (unsigned)g.b, sd + g.off); break;  // b: entries that differ from 1
+        case GR_URS: reg_urs_any<V, RB>(v, g.a, sd + g.off); break;
         case GR_CX: reg_cx_any<V, RB>(v, g.a, g.b); break;
+        case GR_DTS:
+            if constexpr (sizeof(R) == 8) {  // (a tangent of 0 multiplies by 1)
+                reg_dts<V, RB, (1ull << (1 << RB)) - 1, R>(v, (const R*)(sd + g.off));
+            }
+            break;
+        case GR_RS:
+            if constexpr (sizeof(R) == 8) {
+                const R* c = (const R*)(sd + g.off);
+                switch (g.a) {
+                case 0: reg_rs<V, RB, 0, R>(v, c); break;
+                case 1: reg_rs<V, RB, 1, R>(v, c); break;
+                case 2: reg_rs<V, RB, 2, R>(v, c); break;
+                default: if constexpr (RB > 3) reg_rs<V, RB, 3, R>(v, c); break;
+                }
+            }
+            break;
         case GR_H: reg_h_any<V, RB>(v, g.a); break;
         case GR_HD:
             reg_h_any<V, RB>(v, g.a);
-#pragma unroll
-            for (int j = 0; j < (1 << RB); ++j)
-                if ((g.b >> j) & 1) v[j] = cmul(sd[g.off + j], v[j]);
+            reg_dt_any<V, RB>(v, (unsigned)g.b, sd + g.off);
             break;
         default: reg_swap_any<V, RB>(v, g.a, g.b); break;
         }
     }
 }
 
-// Tile copies of a register pass: every thread moves exactly 16 chunks of 16
-// bytes (2^RB amplitudes), chunk k of thread t being tile chunk t + k * blockDim,
-// so the row and in-row offsets advance by compile-time multiples.
-template <typename V>
+// Tile copies of a register pass: every thread moves its 2^RB amplitudes' worth
+// of 16-byte chunks, chunk k of thread t being tile chunk t + k * blockDim, so
+// the row and in-row offsets advance by compile-time multiples.
+template <typename V, int RB>
 __device__ __forceinline__ void rissue_tile(V* tile, const V* __restrict__ psi, uint64_t base, const uint32_t* rowoff,
                                             int L) {
     constexpr int PER = 16 / sizeof(V);
@@ -579,12 +706,12 @@ __device__ __forceinline__ void rissue_tile(V* tile, const V* __restrict__ psi, 
     const int ioff = i0 & ((1 << L) - 1);
     const V* src = psi + base + ioff;
 #pragma unroll 4
-    for (int k = 0; k < 16; ++k) {
+    for (int k = 0; k < (1 << RB) / PER; ++k) {
         const int i = i0 + k * istep;
         cp_async16(tile + swz<V>(i), src + ((uint64_t)rowoff[i >> L] << L));
     }
 }
-template <typename V>
+template <typename V, int RB>
 __device__ __forceinline__ void rstore_tile(const V* tile, V* __restrict__ psi, uint64_t base, const uint32_t* rowoff,
                                             int L) {
     constexpr int PER = 16 / sizeof(V);
@@ -592,7 +719,7 @@ __device__ __forceinline__ void rstore_tile(const V* tile, V* __restrict__ psi, 
     const int ioff = i0 & ((1 << L) - 1);
     V* dst = psi + base + ioff;
 #pragma unroll 4
-    for (int k = 0; k < 16; ++k) {
+    for (int k = 0; k < (1 << RB) / PER; ++k) {
         const int i = i0 + k * istep;
         *(float4*)(dst + ((uint64_t)rowoff[i >> L] << L)) = *(const float4*)(tile + swz<V>(i));
     }
@@ -770,11 +897,9 @@ __device__ __forceinline__ void fill_basis_ct(V* tile, int ix, int i0, int istep
 
 template <typename V, int RB>
 __device__ __forceinline__ void scale_regs(V* v, decltype(V().x) sc) {
+    const V m = vdup<V>(sc);
 #pragma unroll
-    for (int k = 0; k < (1 << RB); ++k) {
-        v[k].x *= sc;
-        v[k].y *= sc;
-    }
+    for (int k = 0; k < (1 << RB); ++k) v[k] = vmul(m, v[k]);
 }
 
 // Per-tile fold of every diagonal run of the pass for tile t.
@@ -817,7 +942,7 @@ __device__ __forceinline__ void fold_diags(const PassDev& P, const unsigned char
 // return the amplitudes are in registers in the last layout (Lg).  issue /
 // store move a tile between the state and shared memory; finish applies the
 // pass's write-back scale and puts the registers back into the tile.
-template <bool TC>
+template <bool TC, int RBT>
 struct InterpOps {
     // tiles move through shared memory (the compiled passes may load their
     // first layout and store their last straight to and from registers)
@@ -825,16 +950,17 @@ struct InterpOps {
     template <typename V>
     static __device__ __forceinline__ void issue(V* tile, const V* __restrict__ psi, uint64_t base,
                                                  const uint32_t* rowoff, int L, const PassDev&) {
-        rissue_tile(tile, psi, base, rowoff, L);
+        rissue_tile<V, RBT>(tile, psi, base, rowoff, L);
     }
     template <typename V>
     static __device__ __forceinline__ void store(const V* tile, V* __restrict__ psi, uint64_t base,
                                                  const uint32_t* rowoff, int L) {
-        rstore_tile(tile, psi, base, rowoff, L);
+        rstore_tile<V, RBT>(tile, psi, base, rowoff, L);
     }
     template <typename V, typename R, int RB>
-    static __device__ __forceinline__ void finish(V* v, V* tile, const PassDev& P, const RegLayout<V, RB>& Lg,
-                                                  TcCtx& T) {
+    static __device__ __forceinline__ void finish(V* v, V* tile, const PassDev& P, RegLayout<V, RB>& Lg, TcCtx& T) {
+#pragma unroll
+        for (int b = 0; b < RB; ++b) Lg.sbit[b] = swz<V>(P.fmask[b]);
         if constexpr (TC && sizeof(R) == 4 && RB == 5) {
             if (P.tc_k) {  // the tile's norm as loaded: scale = sqrt(in / out)
                 warp_norm_to<RB>((const float2*)v, T.nout);
@@ -845,12 +971,7 @@ struct InterpOps {
             }
         }
         if (P.scale != 1.0) {
-            const R sc = (R)P.scale;
-#pragma unroll
-            for (int k = 0; k < (1 << RB); ++k) {
-                v[k].x *= sc;
-                v[k].y *= sc;
-            }
+            scale_regs<V, RB>(v, (R)P.scale);
         }
         // each warp writes back the positions it read last, which no other
         // warp reads: the caller's barrier before the store orders the rest
@@ -859,7 +980,7 @@ struct InterpOps {
     template <typename V, typename R, int RB>
     static __device__ __forceinline__ void tile(V* v, V* tile, const PassDev& P, const unsigned char* stage,
                                                 const uint64_t* fold, RegLayout<V, RB>& Lg, const double2* ttab,
-                                                TcCtx& T) {
+                                                TcCtx& T, const V* = nullptr) {
     const int m = P.m, tb = m - RB, no = P.nother;
     const OpDev* ops = (const OpDev*)stage;
     const int* rpos = nullptr;
@@ -874,6 +995,8 @@ struct InterpOps {
             // writers: the warp's own lanes when the remap keeps every warp's
             // amplitudes within the warp (nrec = 1), else the whole block
             if (in_regs) {
+#pragma unroll
+                for (int b = 0; b < RB; ++b) Lg.sbit[b] = swz<V>(op.wmask[b]);
                 reg_write<V, RB>(v, tile, Lg);
                 if (op.nrec == 1) __syncwarp();
                 else __syncthreads();
@@ -928,10 +1051,12 @@ struct InterpOps {
 // columns per group of 128 threads for the whole kernel; every wait on the
 // tensor cores is bounded (expiry: *err = 1, the group skips its remaining
 // products, the TMEM is still freed).
+// tab: the gate data (matrices, tables) of a compiled pass, a kernel parameter.
 template <typename R, int RB, class Ops, bool TC = false>
 __device__ __forceinline__ void rpass_body(typename CT<R>::V* __restrict__ psi, int n,
                                            const PassDev* __restrict__ pdp, const unsigned char* __restrict__ blob,
-                                           const PassLayout& lay, int* __restrict__ err) {
+                                           const PassLayout& lay, int* __restrict__ err,
+                                           const typename CT<R>::V* tab = nullptr) {
     using V = typename CT<R>::V;
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ PassDev P;
@@ -941,6 +1066,7 @@ __device__ __forceinline__ void rpass_body(typename CT<R>::V* __restrict__ psi, 
     __shared__ __align__(8) uint64_t s_mbar[4];
     __shared__ int s_abort[4];
     __shared__ float s_norm[2][16];  // per warp: tile norm in / out (passes with tensor-core blocks)
+    pdl_trigger();
     {
         const int* src = (const int*)pdp;
         int* dst = (int*)&P;
@@ -992,12 +1118,13 @@ __device__ __forceinline__ void rpass_body(typename CT<R>::V* __restrict__ psi, 
     if (tcp) tc::fence_after();
     TcCtx T{tcp ? s_tmem : 0u, s_mbar, s_abort, err, 0u, s_norm[0], s_norm[1]};
     const OpDev* ops = (const OpDev*)stage;
-    if (threadIdx.x == 0)
+    if (threadIdx.x == 0 && nd)
         for (int i = 0; i < P.nops; ++i)
             if (ops[i].kind == OP_DIAG) dofs[ops[i].ord] = ops[i].diag_off;
     const uint64_t ntiles = 1ull << (n - m);
     auto tile_base = [&](uint64_t t) { return table_base(tbase, t, L); };
     int cur = 0;
+    pdl_wait();  // everything above read the plan only
     if constexpr (!Ops::kDirectLoad) {
         if (lay.nbuf == 2 && (uint64_t)blockIdx.x < ntiles) {
             Ops::template issue<V>(tiles[0], psi, tile_base(blockIdx.x), rowoff, L, P);
@@ -1036,7 +1163,7 @@ __device__ __forceinline__ void rpass_body(typename CT<R>::V* __restrict__ psi, 
             fold_diags<R>(P, stage, fold, dofs, t);
             if constexpr (Ops::kDirectLoad) __syncthreads();
         }
-        Ops::template tile<V, R, RB>(v, tile, P, stage, fold, Lg, sizeof(R) == 8 ? ttab : nullptr, T);
+        Ops::template tile<V, R, RB>(v, tile, P, stage, fold, Lg, sizeof(R) == 8 ? ttab : nullptr, T, tab);
         Ops::template finish<V, R, RB>(v, tile, P, Lg, T);
         if constexpr (Ops::kDirectStore) {
             // the last layout straight from registers to global memory
@@ -1062,7 +1189,7 @@ __global__ void __launch_bounds__(MAXT, MINB) k_rpass(typename CT<R>::V* __restr
                                                   const PassDev* __restrict__ pdp,
                                                   const unsigned char* __restrict__ blob, const PassLayout lay,
                                                   int* __restrict__ err) {
-    rpass_body<R, RB, InterpOps<TC>, TC>(psi, n, pdp, blob, lay, err);
+    rpass_body<R, RB, InterpOps<TC, RB>, TC>(psi, n, pdp, blob, lay, err);
 }
 #endif
 

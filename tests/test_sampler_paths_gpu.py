@@ -9,7 +9,7 @@ import pytest
 import oracle
 import paper_2504_03967_gb300 as S
 import workloads as W
-from gpu_util import BAND, compare_samples
+from tests.gpu_util import BAND, compare_samples
 
 pytestmark = pytest.mark.gpu
 
