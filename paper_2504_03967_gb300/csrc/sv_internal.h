@@ -329,15 +329,11 @@ int device_sms();
 
 // Write a deferred sv_init_basis to the state (no-op when none is pending).
 int flush_init(sv_state* h);
-void used_fields(const sv_gate* gates, size_t count, std::vector<sv_gate>* out);
-uint64_t plan_key(const sv_state* h, const std::vector<sv_gate>& recs, const sv_options* opt);
-bool same_records(const std::vector<sv_gate>& a, const std::vector<sv_gate>& b);
 
 // The body of sv_apply_circuit after validation: plan and launch on h's stream.
-// cache_key != 0: keep the plan under that key (see PlanCache).
-// recs: the used fields of the records (see used_fields), kept with a cached plan.
+// keep: put the plan into h's PlanCache.
 int apply_canonical(sv_state* h, const sv_gate* gates, size_t count, const std::vector<CGate>& cg,
-                    const sv_options* opt, uint64_t cache_key = 0, const std::vector<sv_gate>* recs = nullptr);
+                    const sv_options* opt, bool keep = false);
 
 // Recent plans of a handle: the same gate records, options and qubit map
 // give the same plan, so a repeated apply skips validation, planning and
@@ -350,10 +346,14 @@ struct CachedPlan {
     sv_options last_opts;
     uint64_t stamp;
     std::vector<std::string> jit_srcs;  // compiled-kernel sources of its passes (filled on first launch)
-    std::vector<sv_gate> recs;          // the used fields of the circuit's gate records (compared on a hit)
+    std::vector<sv_gate> recs;          // what the plan is for: the gate records, options and qubit map (plan_matches)
+    sv_options key_opts;
+    bool key_has_opts;
+    bool key_permuted;
+    int key_perm[64];
 };
 struct PlanCache {
-    std::vector<std::pair<uint64_t, CachedPlan>> entries;  // small: linear search, least recently used evicted
+    std::vector<CachedPlan> entries;  // small: linear search, least recently used evicted
     uint64_t clock = 0;
 };
 constexpr int kPlanCacheEntries = 8;
