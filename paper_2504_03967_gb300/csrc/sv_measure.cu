@@ -690,7 +690,8 @@ __global__ void __launch_bounds__(256) k_sample(const V* __restrict__ psi, int b
 // warp-wide FP64 instruction costs 78 clocks here (done by all lanes, these
 // were 120 of 140 us); block CDF entries are compared as integers (finite
 // doubles >= 0 order as their bits).  10^5 shots of a 28-qubit state with the
-// whole block rescanned by a warp per shot: 339 us.
+// whole block rescanned by a warp per shot: 339 us (shots and <Z> 787 us, now
+// 501).
 __global__ void __launch_bounds__(256) k_sample_quarter(const float2* __restrict__ psi, const double* __restrict__ cdf,
                                                         uint64_t nblocks, const float2* __restrict__ quart, int G,
                                                         uint64_t shots, uint64_t seed, uint64_t* __restrict__ out) {
@@ -834,7 +835,7 @@ __global__ void __launch_bounds__(256) k_guide(const uint64_t* __restrict__ fine
 // compares alone were 1.1 ms of the example below): three random 32-byte
 // sectors of L2 per shot (guide, table, table) against a warp's search and
 // rescan of 32 amplitudes.  QCrank read-out of 2^20 amplitudes, 4.9 10^7 shots:
-// one warp per shot took 41.4 ms.
+// one warp per shot took 41.4 ms, this 0.63 ms and its tables 0.05.
 template <typename V, bool PERM>
 __global__ void __launch_bounds__(256) k_sample_dense(const V* __restrict__ psi, const double* __restrict__ cdf, int n,
                                                       const uint64_t* __restrict__ fine,
