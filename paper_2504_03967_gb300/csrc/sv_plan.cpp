@@ -86,7 +86,7 @@ void make_canonical(const sv_gate& g, CGate* c) {
 struct Block {
     std::vector<int> qubits;  // sorted
     std::vector<cd> mat;
-    std::vector<CGate> seq;   // the gates multiplied into mat, in order
+    std::vector<const CGate*> seq;  // its gates, in order (they belong to the caller's list)
     int ngates = 0;
     bool active() const { return !qubits.empty(); }
     int pos(int q) const {
@@ -257,29 +257,28 @@ bool gate_sequence(const Block& B, std::vector<GateRec>* recs, std::vector<cd>* 
     recs->clear();
     data->clear();
     const int k = (int)B.qubits.size(), D = 1 << k;
-    std::vector<CGate> seq;
+    std::vector<const CGate*> seq;
+    std::vector<CGate> own;  // the split gates
     seq.reserve(B.seq.size() * 3);
-    for (const CGate& g : B.seq) {
+    if (split_u3) own.reserve(B.seq.size() * 3);
+    for (const CGate* gp : B.seq) {
+        const CGate& g = *gp;
         if (split_u3 && g.type == SV_U3) {
             sv_gate e;
             memset(&e, 0, sizeof(e));
             e.nq = 1;
             e.q[0] = (uint32_t)g.q[0];
-            CGate c;
-            e.type = SV_P;
-            e.p[0] = g.p[2];
-            make_canonical(e, &c);
-            seq.push_back(c);
-            e.type = SV_RY;
-            e.p[0] = g.p[0];
-            make_canonical(e, &c);
-            seq.push_back(c);
-            e.type = SV_P;
-            e.p[0] = g.p[1];
-            make_canonical(e, &c);
-            seq.push_back(c);
+            const uint32_t types[3] = {SV_P, SV_RY, SV_P};
+            const double angles[3] = {g.p[2], g.p[0], g.p[1]};
+            for (int t = 0; t < 3; ++t) {
+                e.type = types[t];
+                e.p[0] = angles[t];
+                own.emplace_back();
+                make_canonical(e, &own.back());
+                seq.push_back(&own.back());
+            }
         } else {
-            seq.push_back(g);
+            seq.push_back(gp);
         }
     }
     auto posmask = [&](const CGate& g) {
@@ -304,7 +303,7 @@ bool gate_sequence(const Block& B, std::vector<GateRec>* recs, std::vector<cd>* 
         if (!dpend) return;
         // a = the positions the table depends on: entry j equals entry j & a
         recs->push_back(GateRec{GR_DT, dep, 0, (int)data->size()});
-        for (int j = 0; j < D; ++j) data->push_back(std::polar(1.0, ph[j]));
+        for (int j = 0; j < D; ++j) data->push_back(cd(ph[j], 0.0));  // angles until finish_tables
         std::fill(ph.begin(), ph.end(), 0.0);
         dpend = false;
         dep = 0;
@@ -313,7 +312,7 @@ bool gate_sequence(const Block& B, std::vector<GateRec>* recs, std::vector<cd>* 
     std::vector<char> used(N, 0);
     for (int i = 0; i < N; ++i) {
         if (used[i]) continue;
-        const CGate& g = seq[i];
+        const CGate& g = *seq[i];
         if (g.kind == GK_DIAG) {
             add_diag(g);
             continue;
@@ -344,10 +343,10 @@ bool gate_sequence(const Block& B, std::vector<GateRec>* recs, std::vector<cd>* 
             int blocked = 1 << p;
             for (int j = i + 1; j < N && blocked != D - 1; ++j) {
                 if (used[j]) continue;
-                const int pm = posmask(seq[j]);
-                if (seq[j].kind == GK_DIAG) {
+                const int pm = posmask(*seq[j]);
+                if (seq[j]->kind == GK_DIAG) {
                     if (!(pm & blocked)) {
-                        add_diag(seq[j]);
+                        add_diag(*seq[j]);
                         used[j] = 1;
                     }
                 } else {
@@ -373,12 +372,23 @@ bool gate_sequence(const Block& B, std::vector<GateRec>* recs, std::vector<cd>* 
     return (int)recs->size() <= kMaxGateRecs && (int)data->size() <= kMaxGateData;
 }
 
+// The tables' entries from their angles (left until the planner has chosen the
+// block's form: it weighs four per block and keeps one).
+void finish_tables(HostOp* op) {
+    for (const GateRec& g : op->recs)
+        if (g.kind == GR_DT)
+            for (int j = 0; j < (1 << op->qubits.size()); ++j) {
+                cd& e = op->gdata[(size_t)g.off + j];
+                e = std::polar(1.0, e.real());
+            }
+}
+
 // A block's gate sequence: the cheaper of the plain form and, when the block
 // holds U3 gates, the form with each U3 split into P RY P.
 bool best_gate_sequence(const Block& B, std::vector<GateRec>* recs, std::vector<cd>* data) {
     const bool ok = gate_sequence(B, recs, data, false);
     bool u3 = false;
-    for (const CGate& g : B.seq) u3 |= g.type == SV_U3;
+    for (const CGate* g : B.seq) u3 |= g->type == SV_U3;
     if (!u3) return ok;
     std::vector<GateRec> r2;
     std::vector<cd> d2;
@@ -847,8 +857,7 @@ void greedy_pass(int n, int dtype, const std::vector<CGate>& gates, const std::v
                 op.kind = OP_DENSE;
                 op.tc = true;
                 tc_bytes += 2 * tc16_bytes(kb);
-                if (form_matrices) op.mat = block_matrix(B.qubits, B.seq);
-                else op.seq = B.seq;
+                op.from = B.seq;
                 op.recs.clear();
                 op.gdata.clear();
             } else if (seq && (seq_cost <= dense_cost(kb) || (kb > kRegDenseMaxK && po.pass_kernel != 1))) {
@@ -857,13 +866,12 @@ void greedy_pass(int n, int dtype, const std::vector<CGate>& gates, const std::v
                 // register kernel's dense limit stay gate sequences, which
                 // keeps the pass on the register kernel)
                 op.kind = OP_GATES;
-                op.seq = B.seq;
+                op.from = B.seq;
             } else {
                 op.kind = OP_DENSE;
                 // (the shared-memory kernel's 3xTF32 path also takes 3-qubit blocks)
                 op.tc = po.tensor == 0 && dtype == SV_C64 && kb >= kMinTcK && po.pass_kernel == 1;
-                if (form_matrices) op.mat = block_matrix(B.qubits, B.seq);
-                else op.seq = B.seq;
+                op.from = B.seq;
                 op.recs.clear();
                 op.gdata.clear();
             }
@@ -906,7 +914,7 @@ void greedy_pass(int n, int dtype, const std::vector<CGate>& gates, const std::v
                     B.qubits = u;
                 }
                 if (inB || widen) {
-                    B.seq.push_back(g);
+                    B.seq.push_back(&g);
                     B.ngates++;
                 } else {
                     diag_add(&D, n, g);
@@ -935,7 +943,7 @@ void greedy_pass(int n, int dtype, const std::vector<CGate>& gates, const std::v
                 std::sort(u.begin(), u.end());
             }
             B.qubits = u;
-            B.seq.push_back(g);
+            B.seq.push_back(&g);
             B.ngates++;
         }
         flushB();
@@ -953,6 +961,15 @@ void greedy_pass(int n, int dtype, const std::vector<CGate>& gates, const std::v
             if (ops_cost(alt) < ops_cost(pass.ops)) pass.ops.swap(alt);
         }
     }
+    // the chosen blocks keep their gates, or get their matrix
+    for (HostOp& op : pass.ops) {
+        if (op.kind == OP_DIAG) continue;
+        op.seq.reserve(op.from.size());
+        for (const CGate* g : op.from) op.seq.push_back(*g);
+        std::vector<const CGate*>().swap(op.from);
+        if (op.kind == OP_GATES) finish_tables(&op);
+    }
+    if (form_matrices) form_dense_matrices(&pass);
     *pass_out = std::move(pass);
     deferred_out->swap(deferred);
 }
