@@ -307,7 +307,9 @@ extern "C" int sv_batch_run(int C, const int* n_qubits, const int64_t* gate_offs
         bad[c] = canonicalise(n, gates + gate_offsets[c], (size_t)gate_counts[c], &cg[c], &b) != SV_OK;
         if (bad[c] || n <= small_limit(dt) || !host_plans) return;
         PlanOptions po = resolve_options(n, dt, opt);
-        po.fold_perms = true;  // (never compiled)
+        // (a circuit that leaves the waves compiles its passes with jit = 1, and
+        // compiled passes take no folded permutations)
+        po.fold_perms = po.jit < 0;
         if (po.rb != reg_bits(dt)) {
             // the wave kernel holds the wide register count: a wave has warps
             // enough, and fewer passes and remaps (256 20-qubit ansatz circuits:
