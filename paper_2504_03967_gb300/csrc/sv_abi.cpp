@@ -218,6 +218,25 @@ int sync_d2h(sv_handle h, void* host, const void* dev, size_t bytes, const char*
 
 }  // namespace
 
+namespace sv {
+
+void release_scratch(sv_state* h) {
+    for (Scratch* s : {&h->plan_dev, &h->red, &h->out_dev, &h->err, &h->perm_tmp, &h->aux, &h->lcdf, &h->fine}) {
+        if (s->ptr) cudaFree(s->ptr);
+        *s = Scratch{};
+    }
+    if (h->host_pin.ptr) cudaFreeHost(h->host_pin.ptr);
+    h->host_pin = Scratch{};
+    delete h->plans;
+    h->plans = nullptr;
+    for (cudaEvent_t e : h->ev_pool) cudaEventDestroy(e);
+    h->ev_pool.clear();
+    if (h->upload_ev) cudaEventDestroy(h->upload_ev);
+    h->upload_ev = nullptr;
+}
+
+}  // namespace sv
+
 extern "C" {
 
 int sv_version(void) { return 100; }
@@ -264,18 +283,7 @@ int sv_free(sv_handle h) {
     if (!h) return SV_OK;
     cudaStreamSynchronize(h->stream);
     if (h->owned && h->amps) cudaFree(h->amps);
-    if (h->plan_dev.ptr) cudaFree(h->plan_dev.ptr);
-    if (h->red.ptr) cudaFree(h->red.ptr);
-    if (h->out_dev.ptr) cudaFree(h->out_dev.ptr);
-    if (h->err.ptr) cudaFree(h->err.ptr);
-    if (h->perm_tmp.ptr) cudaFree(h->perm_tmp.ptr);
-    if (h->aux.ptr) cudaFree(h->aux.ptr);
-    if (h->lcdf.ptr) cudaFree(h->lcdf.ptr);
-    if (h->fine.ptr) cudaFree(h->fine.ptr);
-    delete h->plans;
-    if (h->host_pin.ptr) cudaFreeHost(h->host_pin.ptr);
-    for (cudaEvent_t e : h->ev_pool) cudaEventDestroy(e);
-    if (h->upload_ev) cudaEventDestroy(h->upload_ev);
+    release_scratch(h);
     cudaGetLastError();
     delete h;
     return SV_OK;

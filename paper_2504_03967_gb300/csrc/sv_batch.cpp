@@ -518,10 +518,7 @@ extern "C" int sv_batch_run(int C, const int* n_qubits, const int64_t* gate_offs
         keep.release();
         for (int v = 0; v < kViews; ++v) {
             cudaStreamSynchronize(vs[v]);
-            if (hv[v].red.ptr) cudaFree(hv[v].red.ptr);
-            if (hv[v].perm_tmp.ptr) cudaFree(hv[v].perm_tmp.ptr);
-            if (hv[v].lcdf.ptr) cudaFree(hv[v].lcdf.ptr);
-            if (hv[v].fine.ptr) cudaFree(hv[v].fine.ptr);
+            release_scratch(&hv[v]);
             cudaStreamDestroy(vs[v]);
         }
         cudaEventDestroy(vev);
@@ -594,13 +591,7 @@ extern "C" int sv_batch_run(int C, const int* n_qubits, const int64_t* gate_offs
             memcpy(host_expz + (size_t)order[i] * nmax, tmp.data() + (size_t)i * nmax, sizeof(double) * nmax);
     }
     for (auto& s : slots) {
-        if (s.h.plan_dev.ptr) cudaFree(s.h.plan_dev.ptr);
-        if (s.h.red.ptr) cudaFree(s.h.red.ptr);
-        if (s.h.fine.ptr) cudaFree(s.h.fine.ptr);
-        if (s.h.err.ptr) cudaFree(s.h.err.ptr);
-        if (s.h.host_pin.ptr) cudaFreeHost(s.h.host_pin.ptr);
-        if (s.h.upload_ev) cudaEventDestroy(s.h.upload_ev);
-        for (cudaEvent_t ev : s.h.ev_pool) cudaEventDestroy(ev);
+        release_scratch(&s.h);
         if (s.buf) cudaFree(s.buf);
         if (s.st) cudaStreamDestroy(s.st);
     }

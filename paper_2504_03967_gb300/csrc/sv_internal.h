@@ -319,6 +319,9 @@ struct QubitMap {
     int phys[40];
 };
 void reset_perm(sv_state* h);
+// Frees every device buffer, pinned buffer and event h holds beside its state,
+// and its plans.
+void release_scratch(sv_state* h);
 QubitMap qubit_map(const sv_state* h);
 
 // Error handling (thread-local message).
