@@ -89,7 +89,6 @@ struct HostOp {
     std::vector<cd> mat;      // dense: the block's 2^k x 2^k matrix, row-major (gates: formed on demand
                               // from seq, see op_matrix)
     std::vector<CGate> seq;   // gates: the block's gates in order
-    std::vector<const CGate*> from;  // the same while the pass is being planned
     std::vector<cd> gdata;    // gates: the records' complex data
     DiagForm diag;            // diag
     std::vector<GateRec> recs;  // gates

@@ -833,7 +833,8 @@ void greedy_pass(int n, int dtype, const std::vector<CGate>& gates, const std::v
     // given order (any order that keeps each qubit's gates in sequence).
     // Blocks keep their qubits and gates; a dense op's matrix is formed
     // when it is emitted, a gate sequence's only if a kernel needs it.
-    auto fuse = [&](const std::vector<int>& order, std::vector<HostOp>* ops_out) {
+    using GateList = std::vector<const CGate*>;
+    auto fuse = [&](const std::vector<int>& order, std::vector<HostOp>* ops_out, std::vector<GateList>* from) {
         Block B;
         DiagForm D;
         D.init(n);
@@ -857,7 +858,6 @@ void greedy_pass(int n, int dtype, const std::vector<CGate>& gates, const std::v
                 op.kind = OP_DENSE;
                 op.tc = true;
                 tc_bytes += 2 * tc16_bytes(kb);
-                op.from = B.seq;
                 op.recs.clear();
                 op.gdata.clear();
             } else if (seq && (seq_cost <= dense_cost(kb) || (kb > kRegDenseMaxK && po.pass_kernel != 1))) {
@@ -866,16 +866,15 @@ void greedy_pass(int n, int dtype, const std::vector<CGate>& gates, const std::v
                 // register kernel's dense limit stay gate sequences, which
                 // keeps the pass on the register kernel)
                 op.kind = OP_GATES;
-                op.from = B.seq;
             } else {
                 op.kind = OP_DENSE;
                 // (the shared-memory kernel's 3xTF32 path also takes 3-qubit blocks)
                 op.tc = po.tensor == 0 && dtype == SV_C64 && kb >= kMinTcK && po.pass_kernel == 1;
-                op.from = B.seq;
                 op.recs.clear();
                 op.gdata.clear();
             }
             ops_out->push_back(std::move(op));
+            from->push_back(std::move(B.seq));
             B = Block();
         };
         int dgates = 0;
@@ -886,6 +885,7 @@ void greedy_pass(int n, int dtype, const std::vector<CGate>& gates, const std::v
             op.diag = D;
             op.ngates = dgates;
             ops_out->push_back(std::move(op));
+            from->emplace_back();
             D.init(n);
             dpend = false;
             dgates = 0;
@@ -949,7 +949,8 @@ void greedy_pass(int n, int dtype, const std::vector<CGate>& gates, const std::v
         flushB();
         flushD();
     };
-    fuse(executed, &pass.ops);
+    std::vector<GateList> from;  // per op, its gates
+    fuse(executed, &pass.ops, &from);
     // A reordering that groups gates by qubit set (each qubit's gates
     // kept in sequence, so the circuit is the same) often needs fewer
     // blocks; keep it when its estimated cost is lower.
@@ -957,16 +958,19 @@ void greedy_pass(int n, int dtype, const std::vector<CGate>& gates, const std::v
         const std::vector<int> reord = cluster_order(gates, executed, kmax);
         if (reord != executed) {
             std::vector<HostOp> alt;
-            fuse(reord, &alt);
-            if (ops_cost(alt) < ops_cost(pass.ops)) pass.ops.swap(alt);
+            std::vector<GateList> alt_from;
+            fuse(reord, &alt, &alt_from);
+            if (ops_cost(alt) < ops_cost(pass.ops)) {
+                pass.ops.swap(alt);
+                from.swap(alt_from);
+            }
         }
     }
     // the chosen blocks keep their gates, or get their matrix
-    for (HostOp& op : pass.ops) {
-        if (op.kind == OP_DIAG) continue;
-        op.seq.reserve(op.from.size());
-        for (const CGate* g : op.from) op.seq.push_back(*g);
-        std::vector<const CGate*>().swap(op.from);
+    for (size_t i = 0; i < pass.ops.size(); ++i) {
+        HostOp& op = pass.ops[i];
+        op.seq.reserve(from[i].size());
+        for (const CGate* g : from[i]) op.seq.push_back(*g);
         if (op.kind == OP_GATES) finish_tables(&op);
     }
     if (form_matrices) form_dense_matrices(&pass);
@@ -979,7 +983,7 @@ void form_dense_matrices(HostPass* hp) {
     for (HostOp& op : hp->ops)
         if (op.kind == OP_DENSE && op.mat.empty() && !op.seq.empty()) {
             op.mat = block_matrix(op.qubits, op.seq);
-            op.seq.clear();
+            std::vector<CGate>().swap(op.seq);
         }
 }
 
@@ -1614,16 +1618,17 @@ bool reg_region(const Plan& p, const HostPass& hp, PassDev* P, const int* loc, s
         }
         OpDev O;
         memset(&O, 0, sizeof(O));
-        if (!rpos.empty()) write_masks(O.wmask);
+        RemapDev M;
+        memset(&M, 0, sizeof(M));
+        if (!rpos.empty()) write_masks(M.wmask);
         rpos = slots;
         tpos = fresh;
         O.kind = OP_REMAP;
         O.k = r;
         O.nrec = local ? 1 : 0;
         for (int b = 0; b < r; ++b) O.lq[b] = rpos[b];
-        int tp[16];
-        for (int t = 0; t < 16; ++t) tp[t] = t < (int)tpos.size() ? tpos[t] : -1;
-        O.mat_off = (int)pay.put(tp, sizeof(tp));
+        for (int t = 0; t < 16; ++t) M.tpos[t] = t < (int)tpos.size() ? tpos[t] : -1;
+        O.mat_off = (int)pay.put(&M, sizeof(M));
         ops.push_back(O);
     };
     auto slot = [&](int pos) { return (int)(std::find(rpos.begin(), rpos.end(), pos) - rpos.begin()); };

@@ -999,8 +999,9 @@ struct InterpOps {
             // writers: the warp's own lanes when the remap keeps every warp's
             // amplitudes within the warp (nrec = 1), else the whole block
             if (in_regs) {
+                const int* wmask = ((const RemapDev*)(stage + op.mat_off))->wmask;
 #pragma unroll
-                for (int b = 0; b < RB; ++b) Lg.sbit[b] = swz<V>(op.wmask[b]);
+                for (int b = 0; b < RB; ++b) Lg.sbit[b] = swz<V>(wmask[b]);
                 reg_write<V, RB>(v, tile, Lg);
                 if (op.nrec == 1) __syncwarp();
                 else __syncthreads();
@@ -1008,7 +1009,7 @@ struct InterpOps {
                 __syncthreads();
             }
             rpos = op.lq;
-            tpos = (const int*)(stage + op.mat_off);
+            tpos = ((const RemapDev*)(stage + op.mat_off))->tpos;
             reg_layout<V, RB>(Lg, rpos, tpos, tb);
             reg_read<V, RB>(v, tile, Lg);
             if constexpr (TC && sizeof(R) == 4 && RB == 5)
