@@ -799,7 +799,9 @@ __global__ void __launch_bounds__(256) k_fine_cdf(const V* __restrict__ psi, con
     }
     const int lane = threadIdx.x & 31;
     const uint64_t warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
-    const double S = cdf[nblocks - 1], scale = S > 0.0 ? kTwo53 / S : 0.0;
+    // (a total too small or too large for the scaled sums to be exact doubles
+    // gets a table of zeros: every shot then takes the rule itself)
+    const double S = cdf[nblocks - 1], scale = S > 1e-280 && S < 1e300 ? kTwo53 / S : 0.0;
     for (uint64_t j = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; j < nblocks; j += warps) {
         const uint64_t x = (j << 5) + lane;
         double inc;

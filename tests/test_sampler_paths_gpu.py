@@ -84,3 +84,19 @@ def test_shots_and_expz_together(n, kind, scale):
         assert np.abs(ez - want).max() <= 1e-12 * cdf[-1]
     finally:
         S.sv_free(h)
+
+
+@pytest.mark.parametrize("scale", [1e-149, 1e-141, 1e-139, 1e149])
+def test_many_shots_far_from_unit_norm(scale):
+    """Totals where 2^53 / S leaves the double range, and both sides of the line
+    at which the table is no longer used."""
+    n = 10
+    h = S.sv_alloc(n, S.C128)
+    try:
+        S.sv_load_state(h, scale * W.random_state(n, 5))
+        cdf = _cdf(h)
+        u = W.uniforms(4 << n, 6)
+        # (the rule and its restatement add 2^n FP64 terms in different orders)
+        compare_samples(S.sv_sample_uniforms(h, u), u, cdf, cdf[-1] * 2.0 ** (n - 52))
+    finally:
+        S.sv_free(h)
