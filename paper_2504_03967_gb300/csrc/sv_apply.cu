@@ -1091,11 +1091,13 @@ cudaError_t launch_batch_small(int dtype, const void* blob_dev, const PlanBlob& 
     int per_sm = 1;
     cudaError_t e;
     if (dtype == SV_C64) {
-        e = cudaFuncSetAttribute(k_batch_small<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        static SmemLimit limit;
+        e = limit.allow((const void*)k_batch_small<float>, (int)smem);
         if (e != cudaSuccess) return e;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_batch_small<float>, kPassThreads, smem);
     } else {
-        e = cudaFuncSetAttribute(k_batch_small<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        static SmemLimit limit;
+        e = limit.allow((const void*)k_batch_small<double>, (int)smem);
         if (e != cudaSuccess) return e;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_batch_small<double>, kPassThreads, smem);
     }
@@ -1190,11 +1192,10 @@ static cudaError_t pass_t(sv_state* h, const void* blob_dev, const PlanBlob& blo
     const int m = (int)hp.tile.size();
     const PassDev* pdh = (const PassDev*)(blob.bytes.data() + blob.pass_off) + pass;
     const PassLayout lay = pass_layout(h->dtype, *pdh);
-    static int attr_bytes = 0;  // dynamic shared memory the kernel is currently allowed
-    if (lay.total > attr_bytes) {
-        cudaError_t e = cudaFuncSetAttribute(k_pass<R, TC>, cudaFuncAttributeMaxDynamicSharedMemorySize, lay.total);
+    static SmemLimit limit;
+    {
+        const cudaError_t e = limit.allow((const void*)k_pass<R, TC>, lay.total);
         if (e != cudaSuccess) return e;
-        attr_bytes = lay.total;
     }
     int per_sm = 1;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_pass<R, TC>, kPassThreads, lay.total);
@@ -1227,12 +1228,10 @@ static cudaError_t rpass_t(sv_state* h, const void* blob_dev, const PlanBlob& bl
     const PassDev* pdh = (const PassDev*)(blob.bytes.data() + blob.pass_off) + pass;
     const PassLayout lay = rpass_layout(h->dtype, *pdh);
     if (lay.total > kMaxDynSmem) return cudaErrorInvalidValue;
-    static int attr_bytes = 0;
-    if (lay.total > attr_bytes) {
-        cudaError_t e = cudaFuncSetAttribute(k_rpass<R, RB, MAXT, MINB, TC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             lay.total);
+    static SmemLimit limit;
+    {
+        const cudaError_t e = limit.allow((const void*)k_rpass<R, RB, MAXT, MINB, TC>, lay.total);
         if (e != cudaSuccess) return e;
-        attr_bytes = lay.total;
     }
     const int threads = 1 << (pdh->m - RB);
     if (threads > MAXT) return cudaErrorInvalidValue;
@@ -1467,7 +1466,8 @@ static cudaError_t wave_t(void* base, const uint64_t* offs, const int* nq, const
                           const WaveItem* items, int nitems, int* head, int* done, int* err, const PassLayout& lay,
                           unsigned limit, cudaStream_t st) {
     int per_sm = 1;
-    cudaError_t e = cudaFuncSetAttribute(k_wave<R, RB, MUX>, cudaFuncAttributeMaxDynamicSharedMemorySize, lay.total);
+    static SmemLimit limit_smem;
+    cudaError_t e = limit_smem.allow((const void*)k_wave<R, RB, MUX>, lay.total);
     if (e == cudaSuccess) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_wave<R, RB, MUX>, 256, lay.total);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) per_sm = 1;
@@ -1583,12 +1583,10 @@ static cudaError_t rpass_tma_t(sv_state* h, const void* blob_dev, const PlanBlob
             CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) !=
         CUDA_SUCCESS)
         return cudaSuccess;  // not expressible: the caller falls back to the copy-based kernel
-    static int attr_bytes = 0;
-    if (lay.total > attr_bytes) {
-        cudaError_t e = cudaFuncSetAttribute(k_rpass_tma<R, RB, MAXT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             lay.total);
+    static SmemLimit limit;
+    {
+        const cudaError_t e = limit.allow((const void*)k_rpass_tma<R, RB, MAXT>, lay.total);
         if (e != cudaSuccess) return e;
-        attr_bytes = lay.total;
     }
     int per_sm = 1;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_rpass_tma<R, RB, MAXT>, threads, lay.total);

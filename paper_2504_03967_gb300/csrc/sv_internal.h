@@ -6,6 +6,7 @@
 
 #include <complex>
 #include <memory>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -327,6 +328,24 @@ QubitMap qubit_map(const sv_state* h);
 int set_error(int code, const std::string& msg);
 int cuda_fail(cudaError_t e, const char* what);
 void count_launch(uint64_t k = 1);
+// The dynamic shared memory a kernel is allowed, per device; it only grows,
+// under a lock, so that a launch on another thread never finds less than it
+// asked for.  (One object per kernel instance.)
+struct SmemLimit {
+    std::mutex mu;
+    int allowed[64] = {};
+    cudaError_t allow(const void* kernel, int bytes) {
+        int dev = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e != cudaSuccess) return e;
+        const bool known = dev >= 0 && dev < 64;
+        std::lock_guard<std::mutex> lk(mu);
+        if (known && bytes <= allowed[dev]) return cudaSuccess;
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        if (e == cudaSuccess && known) allowed[dev] = bytes;
+        return e;
+    }
+};
 // SM count of the current device (cached per device ordinal).
 int device_sms();
 

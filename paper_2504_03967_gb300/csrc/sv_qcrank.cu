@@ -128,12 +128,9 @@ cudaError_t launch_qcrank_decode(const uint64_t* samples, uint64_t shots, int a,
     const size_t smem = sizeof(unsigned int) * J * (size_t)(d + 1);
     if (shots) {
         if (smem <= kHistSmemMax) {
-            static size_t attr = 0;
-            if (smem > 48 * 1024 && smem > attr) {
-                e = cudaFuncSetAttribute(k_qc_hist_smem, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-                if (e != cudaSuccess) return e;
-                attr = smem;
-            }
+            static SmemLimit limit;
+            e = limit.allow((const void*)k_qc_hist_smem, (int)smem);
+            if (e != cudaSuccess) return e;
             // enough CTAs to cover the shots, at most one per SM: every CTA
             // flushes its whole histogram once
             const uint64_t want = (shots + (uint64_t)kHistThreads * 64 - 1) / ((uint64_t)kHistThreads * 64);
@@ -142,7 +139,8 @@ cudaError_t launch_qcrank_decode(const uint64_t* samples, uint64_t shots, int a,
                                                              (unsigned long long*)ones);
         } else if (smem / 2 <= kHist16SmemMax && shots >= (uint64_t)qc_sms() * (kHist16Chunk / 8)) {
             // (fewer shots: too few CTAs for the flushes to pay)
-            e = cudaFuncSetAttribute(k_qc_hist_smem16, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(smem / 2));
+            static SmemLimit limit;
+            e = limit.allow((const void*)k_qc_hist_smem16, (int)(smem / 2));
             if (e != cudaSuccess) return e;
             const uint64_t chunks = (shots + kHist16Chunk - 1) / kHist16Chunk;
             const unsigned grid = (unsigned)std::min<uint64_t>(chunks, (uint64_t)qc_sms());
