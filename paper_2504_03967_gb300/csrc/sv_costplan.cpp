@@ -189,6 +189,7 @@ bool plan_learned(int n, int dtype, const std::vector<CGate>& gates, const std::
     Plan stub;  // register-kernel eligibility of a proposal
     stub.n = n;
     stub.dtype = dtype;
+    stub.rb = base.rb;
     std::vector<BeamNode> nodes(1);
     nodes[0].parent = -1;
     nodes[0].t = 0.0;
@@ -289,8 +290,8 @@ bool plan_learned(int n, int dtype, const std::vector<CGate>& gates, const std::
 }
 
 PlanOptions mlp_plan_options(sv_state* h, const sv_gate* g, size_t count, const std::vector<CGate>& cg,
-                             const std::vector<Mux>* muxes, const PlanOptions& base, uint64_t salt, cudaEvent_t* ev0,
-                             cudaEvent_t* ev1, std::shared_ptr<const Plan>* learned) {
+                             const std::vector<Mux>* muxes, const PlanOptions& base, const PlanOptions& greedy,
+                             uint64_t salt, cudaEvent_t* ev0, cudaEvent_t* ev1, std::shared_ptr<const Plan>* learned) {
     *ev0 = *ev1 = nullptr;
     learned->reset();
     uint64_t key = fnv1a(g, count * sizeof(sv_gate), 1469598103934665603ull);
@@ -302,7 +303,7 @@ PlanOptions mlp_plan_options(sv_state* h, const sv_gate* g, size_t count, const 
     if (it == g_cache.end()) {
         std::vector<PlanOptions> ranked;
         std::vector<double> rms;
-        if (!rank_options(h->n, h->dtype, cg, muxes, base, &ranked, &rms)) return base;  // no model: greedy
+        if (!rank_options(h->n, h->dtype, cg, muxes, base, &ranked, &rms)) return greedy;  // no model
         Choice c;
         auto lp = std::make_shared<Plan>();
         double lms = 0.0;
@@ -315,11 +316,12 @@ PlanOptions mlp_plan_options(sv_state* h, const sv_gate* g, size_t count, const 
             c.trial.push_back(ranked[i]);
             c.pred.push_back(rms[i]);
         }
-        c.trial.push_back(base);
+        c.trial.push_back(greedy);
         double gms = -1.0;  // the greedy plan's prediction, where the ranking had its options
         for (size_t i = 0; i < ranked.size(); ++i)
-            if (ranked[i].k_max == base.k_max && ranked[i].tile_m == base.tile_m && ranked[i].tensor == base.tensor &&
-                ranked[i].pass_kernel == base.pass_kernel && ranked[i].tc_auto == base.tc_auto)
+            if (ranked[i].k_max == greedy.k_max && ranked[i].tile_m == greedy.tile_m && ranked[i].rb == greedy.rb &&
+                ranked[i].tensor == greedy.tensor && ranked[i].pass_kernel == greedy.pass_kernel &&
+                ranked[i].tc_auto == greedy.tc_auto)
                 gms = rms[i];
         c.pred.push_back(gms);
         c.measured.assign(c.trial.size(), -1.0);
@@ -352,6 +354,13 @@ PlanOptions mlp_plan_options(sv_state* h, const sv_gate* g, size_t count, const 
 
 using namespace sv;
 
+// The candidates' options of a call that names nothing but the planner.
+static PlanOptions cost_model_base(int n, sv_dtype dt) {
+    sv_options o{};
+    o.planner = SV_PLAN_MLP;
+    return resolve_options(n, dt, &o);
+}
+
 extern "C" int sv_cost_model_choose(int n, sv_dtype dt, const sv_gate* gates, size_t count, sv_options* chosen,
                                     double* predicted_ms) {
     if (!chosen || !predicted_ms || (count && !gates)) return set_error(SV_EINVAL, "bad arguments");
@@ -361,8 +370,7 @@ extern "C" int sv_cost_model_choose(int n, sv_dtype dt, const sv_gate* gates, si
     size_t bad = 0;
     if (canonicalise(n, gates, count, &cg, &bad) != SV_OK)
         return set_error(SV_EINVAL, "invalid gate record at index " + std::to_string(bad));
-    PlanOptions base = resolve_options(n, dt, nullptr);
-    base.rb = reg_bits(dt);  // the candidates are compiled passes
+    const PlanOptions base = cost_model_base(n, dt);
     std::vector<PlanOptions> ranked;
     std::vector<double> rms;
     if (!rank_options(n, dt, cg, nullptr, base, &ranked, &rms)) return set_error(SV_EINVAL, "no cost model loaded");
@@ -389,8 +397,7 @@ extern "C" int sv_cost_model_judged(int n, sv_dtype dt, const sv_gate* gates, si
                                     double* measured_ms) {
     if (!out || (count && !gates)) return set_error(SV_EINVAL, "bad arguments");
     uint64_t key = fnv1a(gates, count * sizeof(sv_gate), 1469598103934665603ull);
-    PlanOptions base = resolve_options(n, dt, nullptr);
-    base.rb = reg_bits(dt);  // the candidates are compiled passes
+    const PlanOptions base = cost_model_base(n, dt);
     const int meta[3] = {n, (int)dt, base.tensor};
     key = fnv1a(meta, sizeof(meta), key);
     std::lock_guard<std::mutex> lk(g_mu);

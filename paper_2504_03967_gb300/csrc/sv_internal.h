@@ -228,10 +228,12 @@ bool register_pass_eligible(const Plan& p, const HostPass& hp);
 // Options for an apply under SV_PLAN_MLP; ev0/ev1 receive events to record
 // around the passes when the judge times this call (else nullptr).
 // *learned (may stay null): the model's per-pass plan to run instead of
-// plan_greedy with the returned options.
+// plan_greedy with the returned options.  base: the candidates' options;
+// greedy: what the same call plans with SV_PLAN_GREEDY, the judge's yardstick
+// and the answer without a model.
 PlanOptions mlp_plan_options(sv_state* h, const sv_gate* g, size_t count, const std::vector<CGate>& cg,
-                             const std::vector<Mux>* muxes, const PlanOptions& base, uint64_t salt, cudaEvent_t* ev0,
-                             cudaEvent_t* ev1, std::shared_ptr<const Plan>* learned);
+                             const std::vector<Mux>* muxes, const PlanOptions& base, const PlanOptions& greedy,
+                             uint64_t salt, cudaEvent_t* ev0, cudaEvent_t* ev1, std::shared_ptr<const Plan>* learned);
 
 // Multiplexor pass (PassDev::rmode == kRmodeMux): the region is MuxDev
 // followed by one angle table per target: 2^nc entries of the state's real

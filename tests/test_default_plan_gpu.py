@@ -1,0 +1,43 @@
+"""The default plan of small states (half the registers, narrower tiles) as the
+calls that compare, report and time plans see it."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+import paper_2504_03967_gb300 as S
+import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+SIZES = [(S.C64, 9), (S.C64, 13), (S.C64, 16), (S.C64, 19), (S.C64, 21), (S.C128, 9), (S.C128, 12), (S.C128, 16),
+         (S.C128, 18), (S.C128, 20)]
+
+
+def widths(h, g, **opts):
+    S.sv_init_basis(h, 0)
+    S.sv_apply_circuit(h, g, **opts)
+    p = S.sv_last_plan(h)
+    return p["k_max"], p["tile_m"]
+
+
+@pytest.mark.parametrize("dtype,n", SIZES)
+def test_cost_model_planner_is_judged_against_the_default_plan(dtype, n):
+    """Without a model SV_PLAN_MLP runs the default plan; with one the judge's
+    last trial of every round is the default plan."""
+    g = W.random_u3_cx(n, 3, 7)
+    h = S.sv_alloc(n, dtype)
+    try:
+        S.sv_cost_model_unload()
+        default = widths(h, g)
+        assert widths(h, g, planner=S.PLAN_MLP) == default
+        rng = np.random.default_rng(1)
+        X = rng.uniform(0, 1, size=(64, S.sv_feature_count())).astype(np.float32)
+        S.sv_cost_model_train(X, np.exp(X[:, 0]), epochs=50, lr=3e-3, seed=1)
+        seen = [widths(h, g, planner=S.PLAN_MLP)]
+        T = len(S.sv_cost_model_last_trials(16)["predicted_ms"])
+        seen += [widths(h, g, planner=S.PLAN_MLP) for _ in range(2 * T - 1)]
+        assert T > 1 and seen[T - 1] == seen[2 * T - 1] == default
+    finally:
+        S.sv_cost_model_unload()
+        S.sv_free(h)
