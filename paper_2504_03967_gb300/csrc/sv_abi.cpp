@@ -691,7 +691,8 @@ int launch_plan(sv_state* h, const Plan& plan, const PlanBlob& blob, bool rec, c
         if (rec && e1) {
             cudaEventRecord(e1, h->stream);
             const PassDev* pd = (const PassDev*)(blob.bytes.data() + blob.pass_off) + p;
-            h->rec_feat.push_back(pass_features(h->n, h->dtype, plan.passes[p], plan.tensor == 0, pd->rmode == 1 || pd->rmode == 2));
+            h->rec_feat.push_back(pass_features(h->n, h->dtype, plan.passes[p], plan.tensor == 0,
+                                                pd->rmode == 1 || pd->rmode == 2 ? pd->rb : 0));
         }
     }
     if (judge1) cudaEventRecord(judge1, h->stream);

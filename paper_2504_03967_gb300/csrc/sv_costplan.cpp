@@ -116,7 +116,7 @@ bool rank_options(int n, int dtype, const std::vector<CGate>& gates, const std::
         plan_greedy(n, dtype, gates, cands[c], &p, muxes);
         for (HostPass& hp : p.passes) {
             const std::vector<float> f =
-                pass_features(n, dtype, hp, cands[c].tensor == 0, register_pass_eligible(p, hp));
+                pass_features(n, dtype, hp, cands[c].tensor == 0, register_pass_eligible(p, hp) ? p.rb : 0);
             feat.insert(feat.end(), f.begin(), f.end());
             owner.push_back((int)c);
         }
@@ -213,7 +213,7 @@ bool plan_learned(int n, int dtype, const std::vector<CGate>& gates, const std::
                 greedy_pass(n, dtype, gates, mx, cands[c], nodes[b].rem, &pr.hp, &pr.rem, false);
                 const bool mux_pass = !pr.hp.mux.empty();
                 const std::vector<float> f = pass_features(n, dtype, pr.hp, cands[c].tc_auto != 0,
-                                                           mux_pass ? false : register_pass_eligible(stub, pr.hp));
+                                                           !mux_pass && register_pass_eligible(stub, pr.hp) ? stub.rb : 0);
                 feat.insert(feat.end(), f.begin(), f.end());
                 props.push_back(std::move(pr));
                 if (mux_pass) break;  // every candidate proposes the same multiplexor pass

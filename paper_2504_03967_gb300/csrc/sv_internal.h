@@ -218,9 +218,11 @@ void plan_summary(const Plan& p, sv_plan_info* info);
 // Cost-model features of one pass (fixed length kFeatures): qubit count,
 // dtype, tile width, dense blocks per width, diagonal runs, logical gates per
 // type (the paper's one-hot gate-type encoding, App. D.1 Eq. "onehot",
-// summed over the pass), arithmetic and byte volume, and a bias input.
+// summed over the pass), arithmetic and byte volume, the kernel (reg_bits_held:
+// register passes hold 2^that amplitudes per thread, 0 otherwise), and a bias
+// input.
 constexpr int kFeatures = 32;
-std::vector<float> pass_features(int n, int dtype, const HostPass& p, bool tensor_cores, bool register_pass);
+std::vector<float> pass_features(int n, int dtype, const HostPass& p, bool tensor_cores, int reg_bits_held);
 // Whether the register-resident kernel can take the pass (the serialiser's
 // structural conditions; a region too large to stage is checked there).
 bool register_pass_eligible(const Plan& p, const HostPass& hp);

@@ -1088,7 +1088,7 @@ void plan_summary(const Plan& p, sv_plan_info* info) {
     info->bytes_moved = (int64_t)bytes;
 }
 
-std::vector<float> pass_features(int n, int dtype, const HostPass& p, bool tensor_cores, bool register_pass) {
+std::vector<float> pass_features(int n, int dtype, const HostPass& p, bool tensor_cores, int reg_bits_held) {
     std::vector<float> f(kFeatures, 0.0f);
     const int m = (int)p.tile.size();
     f[0] = n / 34.0f;
@@ -1116,7 +1116,8 @@ std::vector<float> pass_features(int n, int dtype, const HostPass& p, bool tenso
     f[13] = (float)p.ops.size() / 16.0f;
     for (int t = 0; t < 14; ++t) f[14 + t] = p.type_count[t] / 16.0f;  // f[14..27]
     f[28] = (float)(ldexp(1.0, n) * (dtype == SV_C64 ? 16.0 : 32.0) / ldexp(1.0, 36));
-    f[29] = register_pass ? 1.0f : 0.0f;  // kernel: register-resident or shared-memory
+    // kernel: shared-memory, register-resident with half the registers, or with all
+    f[29] = reg_bits_held == 0 ? 0.0f : reg_bits_held < reg_bits(dtype) ? 0.5f : 1.0f;
     f[30] = tensor_cores ? ntc / 4.0f : 0.0f;  // blocks on the tensor cores
     f[31] = 1.0f;
     return f;

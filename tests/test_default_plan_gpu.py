@@ -41,3 +41,18 @@ def test_cost_model_planner_is_judged_against_the_default_plan(dtype, n):
     finally:
         S.sv_cost_model_unload()
         S.sv_free(h)
+
+
+@pytest.mark.parametrize("dtype,n,k,m", [(S.C64, 16, 5, 13), (S.C128, 14, 4, 12)])
+def test_recorded_features_tell_the_register_counts_apart(dtype, n, k, m):
+    g = W.random_u3_cx(n, 3, 8)
+    h = S.sv_alloc(n, dtype)
+    try:
+        kernel = []
+        for opts in ({}, dict(k_max=k, tile_m=m), dict(k_max=k, tile_m=m, pass_kernel=1)):
+            S.sv_init_basis(h, 0)
+            S.sv_apply_circuit(h, g, record=1, **opts)
+            kernel.append(set(S.sv_pass_times(h, features=True)[1][:, 29].tolist()))
+        assert kernel == [{0.5}, {1.0}, {0.0}]
+    finally:
+        S.sv_free(h)
