@@ -660,11 +660,10 @@ __device__ __forceinline__ void reg_dt_any(V* v, unsigned mask, const V* __restr
 template <typename V, int RB>
 __device__ __forceinline__ void reg_gates(V* v, const GateRec* __restrict__ recs, int nrec, const V* __restrict__ sd) {
     using R = decltype(V().x);
-    if (nrec <= 0) return;
-    GateRec next = recs[0];
+    // (the next record fetched ahead cost more registers than the fetch: 8-layer
+    // ansatz of 21 qubits 616 us, without 584; random circuit of 14 qubits 196, 183)
     for (int r = 0; r < nrec; ++r) {
-        const GateRec g = next;
-        next = recs[r + 1 < nrec ? r + 1 : r];  // (in flight while this one runs)
+        const GateRec g = recs[r];
         switch (g.kind) {
         case GR_U: reg_u_any<V, RB>(v, g.a, sd[g.off], sd[g.off + 1], sd[g.off + 2], sd[g.off + 3]); break;
         case GR_UR:
