@@ -649,17 +649,38 @@ void drop_small_phases(std::vector<CGate>* g, double eps) {
     g->swap(kept);
 }
 
-// Tile width of plans with small_reg_bits (measured on 8-layer random and
-// ansatz circuits): the whole state while its one CTA is as quick as several
-// passes, then tiles of 32 to 64 threads' worth of CTAs, wider ones as the
-// state fills the GPU.  complex128, bound by the FP64 pipe of the SMs it
-// reaches, keeps about 128 tiles.  0: the wide plan is the faster one (20 and
-// 18 qubits are the last where the small one wins: 257 against 307 us at 20
-// complex64 qubits, 432 against 433 at 21; 517 against 862 at 18 complex128
-// qubits, 2019 against 1802 at 20).
-static int small_tile(int n, int dtype) {
-    if (dtype == SV_C64) return n <= 11 ? n : n <= 15 ? 10 : n <= 17 ? 11 : n <= 20 ? 12 : 0;
-    return n <= 15 ? std::min(n, 10) : n <= 18 ? n - 7 : 0;
+// Shape of the default plans that the interpreting kernels run: false where
+// it is the wide one (13 / 12 qubits per tile, all the registers).
+//
+// Half the registers (small_reg_bits) and a tile that spreads the state over
+// the GPU: the whole state while its one CTA is as quick as several passes,
+// then tiles of 32 to 64 threads' worth of CTAs, wider ones as the state fills
+// the GPU.  complex128, bound by the FP64 pipe of the SMs it reaches, keeps 64
+// to 128 tiles.  Measured on random circuits and ansatz of 2 to 8 layers and
+// the QFT, from 10 / 9 qubits on; 20 and 18 qubits are the last where the small
+// plan wins (microseconds, 8-layer random | ansatz | QFT: 20 complex64 qubits
+// 258 | 371 | 61, wide 292 | 412 | 84; 18 complex128 qubits 442 | 537 | 159,
+// wide 665 | 855 | 233; with 21 and 20 qubits it no longer did).
+//
+// Smaller states run in one CTA of the shared-memory kernel, in blocks of few
+// qubits: forming the matrices of 5-qubit blocks took most of a first call (9
+// complex64 qubits, 8-layer random | ansatz, a call with new angles: 3-qubit
+// blocks 185 | 188, 5-qubit 705 | 1109, half the registers 226 | 247; the same
+// circuit again 26 | 48, 36 | 81, 60 | 72).  A state of 5 complex64 qubits or
+// fewer keeps its one block (5 qubits, ansatz again: 17, in 3-qubit blocks 35).
+struct SmallShape {
+    int rb, k, m;
+};
+static bool small_shape(int n, int dtype, SmallShape* s) {
+    const bool c64 = dtype == SV_C64;
+    if (n <= (c64 ? 9 : 8)) {
+        *s = SmallShape{reg_bits(dtype), c64 ? 3 : 2, n};
+        return !c64 || n > 5;
+    }
+    if (n > (c64 ? 20 : 18)) return false;
+    s->rb = s->k = small_reg_bits(dtype);
+    s->m = c64 ? (n <= 11 ? n : n <= 15 ? 10 : n <= 17 ? 11 : 12) : (n <= 16 ? std::min(n, 10) : n - 7);
+    return true;
 }
 
 PlanOptions resolve_options(int n, int dtype, const sv_options* opt) {
@@ -687,16 +708,16 @@ PlanOptions resolve_options(int n, int dtype, const sv_options* opt) {
     po.k_max = std::max(2, std::min(kMaxK, po.k_max));
     const int mmax = dtype == SV_C64 ? 14 : 13;
     po.rb = reg_bits(dtype);
-    // Plans of default shape that the interpreting kernel will run (never
-    // compiled, or too small to be): half the amplitudes per thread and a tile
-    // that spreads the state over the GPU.
+    // Plans of default shape that the interpreting kernels will run (never
+    // compiled, or too small to be).
+    SmallShape small;
     if (po.planner == SV_PLAN_GREEDY && po.pass_kernel == 0 && po.tensor < 0 && !po.tc_auto &&
-        (po.jit < 0 || (po.jit == 0 && n < kJitAutoMinQubits)) && small_tile(n, dtype) > 0 &&
+        (po.jit < 0 || (po.jit == 0 && n < kJitAutoMinQubits)) && small_shape(n, dtype, &small) &&
         (!opt || (opt->k_max <= 0 && opt->tile_m <= 0))) {
-        po.rb = small_reg_bits(dtype);
-        po.fold_perms = true;
-        po.k_max = po.rb;
-        po.tile_m = small_tile(n, dtype);
+        po.fold_perms = small.rb < po.rb;
+        po.rb = small.rb;
+        po.k_max = small.k;
+        po.tile_m = small.m;
     }
     po.tile_m = std::max(1, std::min(mmax, po.tile_m));
     po.tile_m = std::min(po.tile_m, n);

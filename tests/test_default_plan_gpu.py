@@ -7,6 +7,8 @@ import pytest
 
 import paper_2504_03967_gb300 as S
 import workloads as W
+from tests import gpu_util as U
+from tests.test_small_plans_gpu import circuits
 
 pytestmark = pytest.mark.gpu
 
@@ -56,3 +58,23 @@ def test_recorded_features_tell_the_register_counts_apart(dtype, n, k, m):
         assert kernel == [{0.5}, {1.0}, {0.0}]
     finally:
         S.sv_free(h)
+
+
+@pytest.mark.parametrize("dtype,n", [(S.C64, n) for n in range(2, 11)] + [(S.C128, n) for n in (*range(2, 10), 16, 17)])
+def test_smallest_default_plans_vs_oracle(dtype, n):
+    psi0 = W.random_state(n, 5)
+    for what, g in circuits(n, 3 * n + dtype):
+        U.assert_close(U.run_gpu(n, g, dtype, psi0=psi0), U.run_oracle(n, g, psi0), dtype, "%s n=%d" % (what, n))
+
+
+def test_default_plan_shapes():
+    """Block and tile width on both sides of each line of the rule."""
+    want = {(S.C64, 5): (5, 5), (S.C64, 6): (3, 6), (S.C64, 9): (3, 9), (S.C64, 10): (4, 10), (S.C64, 20): (4, 12),
+            (S.C64, 21): (5, 13), (S.C128, 8): (2, 8), (S.C128, 9): (3, 9), (S.C128, 16): (3, 10), (S.C128, 17): (3, 10),
+            (S.C128, 18): (3, 11), (S.C128, 19): (4, 12)}
+    for (dtype, n), shape in want.items():
+        h = S.sv_alloc(n, dtype)
+        try:
+            assert widths(h, W.random_u3_cx(n, 2, 1)) == shape, (dtype, n)
+        finally:
+            S.sv_free(h)
