@@ -28,21 +28,22 @@ def test_cost_model_planner_is_judged_against_the_default_plan(dtype, n):
     """Without a model SV_PLAN_MLP runs the default plan; with one the judge's
     last trial of every round is the default plan."""
     g = W.random_u3_cx(n, 3, 7)
-    h = S.sv_alloc(n, dtype)
+    S.sv_cost_model_unload()
+    h, h2 = S.sv_alloc(n, dtype), S.sv_alloc(n, dtype)
     try:
-        S.sv_cost_model_unload()
         default = widths(h, g)
         assert widths(h, g, planner=S.PLAN_MLP) == default
         rng = np.random.default_rng(1)
         X = rng.uniform(0, 1, size=(64, S.sv_feature_count())).astype(np.float32)
         S.sv_cost_model_train(X, np.exp(X[:, 0]), epochs=50, lr=3e-3, seed=1)
-        seen = [widths(h, g, planner=S.PLAN_MLP)]
+        seen = [widths(h2, g, planner=S.PLAN_MLP)]
         T = len(S.sv_cost_model_last_trials(16)["predicted_ms"])
-        seen += [widths(h, g, planner=S.PLAN_MLP) for _ in range(2 * T - 1)]
+        seen += [widths(h2, g, planner=S.PLAN_MLP) for _ in range(2 * T - 1)]
         assert T > 1 and seen[T - 1] == seen[2 * T - 1] == default
     finally:
         S.sv_cost_model_unload()
         S.sv_free(h)
+        S.sv_free(h2)
 
 
 @pytest.mark.parametrize("dtype,n,k,m", [(S.C64, 16, 5, 13), (S.C128, 14, 4, 12)])
