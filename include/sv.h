@@ -201,7 +201,9 @@ int sv_qubit_map(sv_handle h, int *map);
 int sv_materialize(sv_handle h);
 
 /* Options the last sv_apply_circuit on h planned with (for SV_PLAN_MLP, the
- * candidate the cost model and its judge picked for that call). */
+ * candidate the cost model and its judge picked for that call).  An apply with
+ * the returned k_max, tile_m, tensor, pass_kernel and jit plans the same way
+ * (not the cost model's own per-pass plan, which has no such options). */
 int sv_last_plan(sv_handle h, sv_options *out);
 
 /* |x>: all amplitudes 0 except a_x = 1.  SV_EINVAL if x >= 2^n.  The write

@@ -709,11 +709,12 @@ PlanOptions resolve_options(int n, int dtype, const sv_options* opt) {
     const int mmax = dtype == SV_C64 ? 14 : 13;
     po.rb = reg_bits(dtype);
     // Plans of default shape that the interpreting kernels will run (never
-    // compiled, or too small to be).
+    // compiled, or too small to be); a caller who names that shape (sv_last_plan,
+    // sv_autotune and the cost model's judge hand it out) gets the same plan.
     SmallShape small;
     if (po.planner == SV_PLAN_GREEDY && po.pass_kernel == 0 && po.tensor < 0 && !po.tc_auto &&
         (po.jit < 0 || (po.jit == 0 && n < kJitAutoMinQubits)) && small_shape(n, dtype, &small) &&
-        (!opt || (opt->k_max <= 0 && opt->tile_m <= 0))) {
+        (!opt || (opt->k_max <= 0 && opt->tile_m <= 0) || (opt->k_max == small.k && opt->tile_m == small.m))) {
         po.fold_perms = small.rb < po.rb;
         po.rb = small.rb;
         po.k_max = small.k;

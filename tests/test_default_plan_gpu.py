@@ -79,3 +79,24 @@ def test_default_plan_shapes():
             assert widths(h, W.random_u3_cx(n, 2, 1)) == shape, (dtype, n)
         finally:
             S.sv_free(h)
+
+
+@pytest.mark.parametrize("dtype,n", SIZES + [(S.C64, 14), (S.C128, 10)])
+def test_reported_options_name_the_plan_that_ran(dtype, n):
+    """sv_last_plan's options, handed back, give the default plan again: the
+    same passes (recorded features) and, bit for bit, the same state."""
+    g = W.random_u3_cx(n, 3, 9)
+    runs = []
+    opts = {}
+    for _ in range(2):
+        h = S.sv_alloc(n, dtype)
+        try:
+            S.sv_load_state(h, W.random_state(n, 2))
+            S.sv_apply_circuit(h, g, record=1, **opts)
+            p = S.sv_last_plan(h)
+            opts = {k: p[k] for k in ("k_max", "tile_m", "tensor", "pass_kernel")}
+            runs.append((opts, S.sv_pass_times(h, features=True)[1], S.sv_store_state(h)))
+        finally:
+            S.sv_free(h)
+    (o1, f1, s1), (o2, f2, s2) = runs
+    assert o1 == o2 and np.array_equal(f1, f2) and np.array_equal(s1, s2)
