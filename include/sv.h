@@ -425,8 +425,9 @@ int sv_feature_count(void);
  * bound) x tile width (11..14 qubits for complex64, 10..13 for complex128,
  * at most n) x, for complex64, tensor cores on or off (blocks of 3..5
  * qubits) x pass kernel (register-resident where it can run, or the
- * shared-memory kernel).  Each candidate runs twice on h's stream and keeps its faster
- * CUDA-event time.  h's amplitudes serve as scratch: their content is
+ * shared-memory kernel); and the default plan, whose widths may be others.
+ * Each candidate runs twice on h's stream and keeps the faster CUDA-event time
+ * of its passes.  h's amplitudes serve as scratch: their content is
  * undefined afterwards.  cache_path (may be NULL) names a JSON-lines file of
  * earlier results, one object per line {"key", "k_max", "tile_m", "tensor",
  * "pass_kernel", "ms"}; the key holds n, dtype, the gate count, a 64-bit FNV-1a hash of the

@@ -517,7 +517,7 @@ int sv_apply_circuit(sv_handle h, const sv_gate* gates, size_t count, const sv_o
 namespace sv {
 
 int apply_canonical(sv_state* h, const sv_gate* gates, size_t count, const std::vector<CGate>& cg,
-                    const sv_options* opt, bool keep) {
+                    const sv_options* opt, bool keep, cudaEvent_t before, cudaEvent_t after) {
     int rc = SV_OK;
     if (cg.empty()) return SV_OK;
     int perm_before[64];  // the map this plan starts from
@@ -625,7 +625,7 @@ int apply_canonical(sv_state* h, const sv_gate* gates, size_t count, const std::
             return launch_plan(h, c.plan, c.blob, opt && opt->record, nullptr, judge1, &c.jit_srcs);
         }
     }
-    return launch_plan(h, plan, blob, opt && opt->record, judge0, judge1);
+    return launch_plan(h, plan, blob, opt && opt->record, judge0 ? judge0 : before, judge1 ? judge1 : after);
 }
 
 int launch_plan(sv_state* h, const Plan& plan, const PlanBlob& blob, bool rec, cudaEvent_t judge0,

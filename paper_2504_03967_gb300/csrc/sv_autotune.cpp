@@ -131,6 +131,21 @@ extern "C" int sv_autotune(sv_handle h, const sv_gate* gates, size_t count, cons
                                c.pass_kernel == o.pass_kernel;
                     if (!dup) cands.push_back(o);
                 }
+    // the plan a call without options runs, where it is not one of these
+    const PlanOptions def = resolve_options(h->n, h->dtype, nullptr);
+    bool have = false;
+    for (const sv_options& c : cands)
+        have |= c.k_max == def.k_max && c.tile_m == def.tile_m && c.tensor == -1 && c.pass_kernel == def.pass_kernel;
+    if (!have) {
+        sv_options o;
+        memset(&o, 0, sizeof(o));
+        o.k_max = def.k_max;
+        o.tile_m = def.tile_m;
+        o.tensor = -1;
+        o.pass_kernel = def.pass_kernel;
+        o.planner = SV_PLAN_GREEDY;
+        cands.push_back(o);
+    }
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     cudaError_t e = cudaEventCreate(&e0);
     if (e == cudaSuccess) e = cudaEventCreate(&e1);
@@ -142,10 +157,12 @@ extern "C" int sv_autotune(sv_handle h, const sv_gate* gates, size_t count, cons
     for (const sv_options& o : cands) {
         double t_best = -1.0;
         for (int rep = 0; rep < 2 && rc == SV_OK; ++rep) {
+            // the events move to the plan's launches (planning it on the host
+            // takes longer than a small state's passes; none: an empty circuit)
             e = cudaEventRecord(e0, h->stream);
-            if (e == cudaSuccess) rc = apply_canonical(h, gates, count, cg, &o);
-            if (rc != SV_OK) break;
             if (e == cudaSuccess) e = cudaEventRecord(e1, h->stream);
+            if (e == cudaSuccess) rc = apply_canonical(h, gates, count, cg, &o, false, e0, e1);
+            if (rc != SV_OK) break;
             if (e == cudaSuccess) e = cudaEventSynchronize(e1);
             float t = 0.f;
             if (e == cudaSuccess) e = cudaEventElapsedTime(&t, e0, e1);

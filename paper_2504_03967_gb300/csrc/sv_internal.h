@@ -357,9 +357,10 @@ int device_sms();
 int flush_init(sv_state* h);
 
 // The body of sv_apply_circuit after validation: plan and launch on h's stream.
-// keep: put the plan into h's PlanCache.
+// keep: put the plan into h's PlanCache.  before, after (optional): events
+// recorded around the plan's launches.
 int apply_canonical(sv_state* h, const sv_gate* gates, size_t count, const std::vector<CGate>& cg,
-                    const sv_options* opt, bool keep = false);
+                    const sv_options* opt, bool keep = false, cudaEvent_t before = nullptr, cudaEvent_t after = nullptr);
 
 // Recent plans of a handle: the same gate records, options and qubit map
 // give the same plan, so a repeated apply skips validation, planning and

@@ -100,3 +100,31 @@ def test_reported_options_name_the_plan_that_ran(dtype, n):
             S.sv_free(h)
     (o1, f1, s1), (o2, f2, s2) = runs
     assert o1 == o2 and np.array_equal(f1, f2) and np.array_equal(s1, s2)
+
+
+@pytest.mark.parametrize("dtype,n", [(S.C64, 8), (S.C64, 14), (S.C64, 17), (S.C128, 8), (S.C128, 14), (S.C128, 17)])
+def test_autotune_times_the_default_plan(dtype, n):
+    """The tuned options are no slower than passing none (best of several
+    calls of each, within their noise)."""
+    torch = pytest.importorskip("torch")
+    g = W.random_u3_cx(n, 6, 3)
+    h = S.sv_alloc(n, dtype)
+    try:
+        tuned, _ = S.sv_autotune(h, g)
+        e0, e1 = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+        best = []
+        for opts in ({}, tuned):
+            t = []
+            for _ in range(12):
+                S.sv_init_basis(h, 0)
+                S.sv_norm(h)
+                torch.cuda.synchronize()
+                e0.record()
+                S.sv_apply_circuit(h, g, **opts)
+                e1.record()
+                e1.synchronize()
+                t.append(e0.elapsed_time(e1))
+            best.append(min(t[2:]))
+        assert best[1] <= 1.15 * best[0] + 0.003, (tuned, best)
+    finally:
+        S.sv_free(h)
