@@ -88,7 +88,7 @@ __device__ __forceinline__ FF ff_allreduce(FF a) {
 // first four exchange steps halves the values a lane keeps, so lane 2e
 // (e < 14) ends with value e summed over all 32 lanes.
 __device__ __forceinline__ void block_stats_c64_full(const float2* __restrict__ psi, uint64_t wid, int lane,
-                                                     double* __restrict__ tot, FF* __restrict__ sbits,
+                                                     double* __restrict__ tot, double* __restrict__ sbits,
                                                      float2* __restrict__ quart) {
     const uint64_t b0 = wid << 10;
     FF p[32];
@@ -142,10 +142,11 @@ __device__ __forceinline__ void block_stats_c64_full(const float2* __restrict__ 
     ff_add(e[0], __shfl_xor_sync(0xffffffffu, e[0].hi, 1), __shfl_xor_sync(0xffffffffu, e[0].lo, 1));
     // value idx: 0 total; 1..5 lane bits 0..4; 6..10 j bits = index bits 5..9; 11..13 quarters
     const int idx = ((lane >> 4) & 1) * 8 + ((lane >> 3) & 1) * 4 + ((lane >> 2) & 1) * 2 + ((lane >> 1) & 1);
-    if (lane == 0) tot[wid] = ff_val(e[0]);
+    const double val = ff_val(e[0]);  // (the same instructions for all of them)
+    if (lane == 0) tot[wid] = val;
     if (!(lane & 1)) {
         if (idx >= 11 && idx < 14 && quart) quart[wid * 4 + (idx - 11)] = make_float2(e[0].hi, e[0].lo);
-        if (idx >= 1 && idx < 11) sbits[(threadIdx.x >> 5) * 10 + idx - 1] = e[0];
+        if (idx >= 1 && idx < 11) sbits[(threadIdx.x >> 5) * 10 + idx - 1] = val;
     }
 }
 constexpr int kBitsGroupLog = 3;  // complex64 bit sums: one record per CTA of k_block_stats (8 blocks)
@@ -162,18 +163,22 @@ __global__ void __launch_bounds__(256) k_block_stats(const V* __restrict__ psi, 
     const int jn = len >= 32 ? len / 32 : 1;
     if constexpr (sizeof(V) == 8) {
         if (bits && blog == 10) {
-            __shared__ FF sbits[80];
+            __shared__ double sbits[80];
             block_stats_c64_full((const float2*)psi, wid, lane, tot, sbits, quart);
             if (nblocks < 8) {  // (one partly filled CTA: a record per block)
                 __syncwarp();
-                if (lane < 10) bits[wid * 10 + lane] = ff_val(sbits[(threadIdx.x >> 5) * 10 + lane]);
+                if (lane < 10) bits[wid * 10 + lane] = sbits[(threadIdx.x >> 5) * 10 + lane];
                 return;
             }
             __syncthreads();  // (nblocks is a multiple of 8: every warp is here)
-            if (threadIdx.x < 10) {
-                FF v = sbits[threadIdx.x];
-                for (int w = 1; w < 8; ++w) ff_add(v, sbits[10 * w + threadIdx.x].hi, sbits[10 * w + threadIdx.x].lo);
-                bits[(uint64_t)blockIdx.x * 10 + threadIdx.x] = ff_val(v);
+            // (in FP64: a float pair would drop what a double still holds.  Lanes
+            // 0..9 add blocks 0..3, lanes 10..19 blocks 4..7)
+            if (threadIdx.x < 32) {
+                const int l = threadIdx.x < 20 ? threadIdx.x : 0, bit = l % 10;
+                const double* src = sbits + (l < 10 ? 0 : 40) + bit;
+                double v = (src[0] + src[10]) + (src[20] + src[30]);
+                v += __shfl_down_sync(0xffffffffu, v, 10);
+                if (threadIdx.x < 10) bits[(uint64_t)blockIdx.x * 10 + threadIdx.x] = v;
             }
             return;
         }
@@ -245,9 +250,8 @@ __global__ void __launch_bounds__(256) k_block_stats(const V* __restrict__ psi, 
 // record-index bit at or above lper selects whole CTAs).  All sums have a
 // fixed order.  Bound by the FP64 pipe (one warp add per 78 clocks and
 // scheduler on this GPU), so the warp sums go through one reduce-scatter (16
-// adds for 16 values) and the bit sums arrive added over 8 blocks in
-// double-float; one CTA per qubit and chunk reading every block's ten sums
-// took 63 us at 2^18 records.
+// adds for 16 values) and the bit sums arrive added over 8 blocks; one CTA per
+// qubit and chunk reading every block's ten sums took 63 us at 2^18 records.
 struct ExpzItem {
     uint64_t blk0;    // first block record of the state
     uint64_t nb;      // its records (a power of two)
