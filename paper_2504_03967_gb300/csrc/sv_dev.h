@@ -40,8 +40,8 @@ enum GateRecKind { GR_U = 0, GR_UR = 1, GR_DT = 2, GR_CX = 3, GR_SWAP = 4, GR_H 
 // GR_HD (register passes only): GR_H on position a followed by the phase table
 // at off with entry mask b (one dispatch for the pair).
 // GR_URS (register passes only): a rotation [[c, -s], [s, c]] on position a as
-// [[1, -t], [t, 1]], t = s / c; (t, t) and (-t, -t) at off, the factor c joins
-// PassDev::scale like GR_H's.  One form for every angle, so circuits of one
+// [[1, -t], [t, 1]], t = s / c; (t, t) and (-t, -t) at off, the factor c
+// (complex64: that of t as rounded) joins PassDev::scale like GR_H's.  One form for every angle, so circuits of one
 // shape share their compiled passes; a rotation with |c| < kMinDeferredCos stays
 // a GR_UR (t would use up the range the deferred factors may take).
 // GR_DTS, GR_RS (complex128 register passes): a phase table without its

@@ -128,3 +128,25 @@ def test_autotune_times_the_default_plan(dtype, n):
         assert best[1] <= 1.15 * best[0] + 0.003, (tuned, best)
     finally:
         S.sv_free(h)
+
+
+@pytest.mark.parametrize("opts", [{}, dict(k_max=5, tile_m=13), dict(jit=1)], ids=["default", "wide", "compiled"])
+def test_rotations_keep_the_norm(opts):
+    """Rotations whose tangent 2 + 0.45 ulp rounds down: with their factor taken
+    from the unrounded cosine each would lose 2 s^2 * 0.45 * 2^-23 of the norm
+    squared, all with one sign.  The rest (the pass's factor rounded once per
+    call, rounding of either sign) is below a quarter of that."""
+    n, calls = 11, 30
+    t = 2.0 + 0.45 * 2.0 ** -22
+    items = [(W.RY, (q,), (2.0 * np.arctan(t),)) for q in range(n)] + [(W.CX, (q, (q + 1) % n), ()) for q in range(n)]
+    g = W.gates_from_list(items)
+    h = S.sv_alloc(n, S.C64)
+    try:
+        S.sv_load_state(h, W.random_state(n, 1))
+        norm0 = S.sv_norm(h)
+        for _ in range(calls):
+            S.sv_apply_circuit(h, g, **opts)
+        drift = 2 * 0.8 * 0.45 * 2.0 ** -23 * n * calls
+        assert abs(S.sv_norm(h) ** 2 / norm0 ** 2 - 1.0) < 0.25 * drift
+    finally:
+        S.sv_free(h)
