@@ -1943,6 +1943,31 @@ bool register_pass_eligible(const Plan& p, const HostPass& hp) {
     return true;
 }
 
+// The factors a plan's register passes multiply their amplitudes by become
+// powers of two, exact in every type, in all passes but the last, which takes
+// what remains: one rounding per amplitude, not one per pass.  (Passes are
+// linear: the state between two of them may be off by a factor of up to
+// sqrt(2).  Tensor-core passes restore their own norm and keep their factor.)
+static void gather_factors(PassDev* pd, size_t count) {
+    auto has = [](const PassDev& P) { return (P.rmode == 1 || P.rmode == 2) && P.tc_k == 0 && P.scale != 1.0; };
+    size_t last = count;
+    for (size_t i = 0; i < count; ++i)
+        if (has(pd[i])) last = i;
+    double rest = 1.0;
+    for (size_t i = 0; i < count && last < count; ++i) {
+        if (!has(pd[i])) continue;
+        const double t = pd[i].scale * rest;
+        if (i == last) {
+            pd[i].scale = t;
+            break;
+        }
+        int e;
+        const double m = std::frexp(std::fabs(t), &e);  // in [1/2, 1)
+        pd[i].scale = std::copysign(std::ldexp(m < 0.70710678 ? 0.5 : 1.0, e), t);
+        rest = t / pd[i].scale;
+    }
+}
+
 void serialise_plans(const std::vector<const Plan*>& plans, PlanBlob* blob) {
     const int dtype = plans.empty() ? SV_C64 : plans[0]->dtype;
     size_t ntc = 0, npass = 0;
@@ -1995,6 +2020,7 @@ void serialise_plans(const std::vector<const Plan*>& plans, PlanBlob* blob) {
             }
             smem_region(p, hp, &P, loc, tcf.data(), &ti, &regions[gpi]);
         }
+        gather_factors(pds.data() + gpi - p.passes.size(), p.passes.size());
     }
     size_t roff = roff0;
     blob->max_region = 0;
