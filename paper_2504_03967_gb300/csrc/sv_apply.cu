@@ -1214,9 +1214,14 @@ static cudaError_t pass_t(sv_state* h, const void* blob_dev, const PlanBlob& blo
 
 // Whether a pass may start before the previous one has finished: its CTAs then
 // find idle SMs (at most one for every two), or fill the GPU anyway and take
-// the places of the previous pass's as they end.  In between they would crowd
-// onto the few SMs the previous pass left idle (20 qubits, 128 CTAs: passes a
-// fifth slower).
+// the places of the previous pass's as they end.  In between they crowd onto
+// the few SMs the previous pass left idle, which heavy passes pay for and light
+// ones do not (8-layer random | ansatz | QFT, microseconds without -> with: 20
+// complex64 qubits, 256 CTAs, 245 -> 275 | 370 -> 387 | 61 -> 59; 17 complex128
+// qubits, 128 CTAs, 292 -> 318 | 402 -> 344 | 110 -> 96).  On this side of the
+// lines: 18 complex64 qubits, 64 CTAs, 160 -> 147 | 263 -> 202 | 52 -> 40; 22,
+// filling the GPU, 916 -> 885 | 1131 -> 1064 | 194 -> 180 (compiled 240 -> 212 |
+// 347 -> 274 | 94 -> 80; of 24 qubits 825 -> 868 | 1100 -> 1038 | 322 -> 320).
 bool pdl_pays(int pass, uint64_t grid, int per_sm) {
     const uint64_t sms = (uint64_t)num_sms();
     return pass > 0 && (2 * grid <= sms || grid == sms * per_sm);

@@ -121,10 +121,12 @@ template <typename V> __device__ __forceinline__ int swz(int i) {
     else return i ^ ((i >> 3) & 7);                                   // 1 amplitude per chunk
 }
 
-// Programmatic dependent launch: a pass kernel lets the next one start as soon
-// as all its CTAs run (pdl_trigger), so that the next pass's staging and tables
-// overlap this pass; before it touches the state it waits for this one to have
-// finished (pdl_wait).  Launched without the attribute both do nothing.
+// Programmatic dependent launch: before a pass kernel touches the state it
+// waits for the previous one to have finished (pdl_wait), then lets the next
+// one start (pdl_trigger), whose staging and tables so overlap this pass.
+// Triggered before the wait, three and more passes held places on the SMs at
+// once (18 complex64 qubits, 8-layer random circuit: 195 us, without early starts
+// 160, so 147).  Launched without the attribute both do nothing.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 
@@ -1070,7 +1072,6 @@ __device__ __forceinline__ void rpass_body(typename CT<R>::V* __restrict__ psi, 
     __shared__ __align__(8) uint64_t s_mbar[4];
     __shared__ int s_abort[4];
     __shared__ float s_norm[2][16];  // per warp: tile norm in / out (passes with tensor-core blocks)
-    pdl_trigger();
     {
         const int* src = (const int*)pdp;
         int* dst = (int*)&P;
@@ -1130,6 +1131,7 @@ __device__ __forceinline__ void rpass_body(typename CT<R>::V* __restrict__ psi, 
     auto tile_base = [&](uint64_t t) { return table_base(tbase, t, L); };
     int cur = 0;
     pdl_wait();  // everything above read the plan only
+    pdl_trigger();
     if constexpr (!Ops::kDirectLoad) {
         if (lay.nbuf == 2 && (uint64_t)blockIdx.x < ntiles) {
             Ops::template issue<V>(tiles[0], psi, tile_base(blockIdx.x), rowoff, L, P);
