@@ -1133,12 +1133,17 @@ int measure_norm(sv_state* h, double* host_out) {
     return SV_OK;
 }
 
-// The table pays once the shots number a quarter of the amplitudes: it reads
-// 8 bytes and writes 12 per amplitude (about 40 us at 2^20 amplitudes), a shot
-// without it takes about 1 ns.  Up to 2^24 amplitudes (200 MB).
+// When the table pays: without it a shot takes 0.9 ns, with it three more
+// launches and two passes over the table's 12 bytes per amplitude come first.
+// Sampling alone, microseconds, table | one warp per shot: 2^15 shots of 14
+// qubits 38 | about 52, of 16 qubits 42 | 51, of 18 qubits 54 | 54; 2^14 of 14 qubits
+// 38 | 34, of 16 qubits 42 | 38; 2^n / 12 shots of 20 qubits 108 | 124, of 24
+// qubits 1023 | 1503, 2^n / 24 of them 108 | 86 and 1006 | 864 (complex128 within
+// 15% of these).  Up to 2^24 amplitudes (200 MB, kept with the handle).
 constexpr int kDenseMaxQubits = 24;
+constexpr uint64_t kDenseMinShots = 1ull << 15;
 static bool dense_shots(int n, int blog, uint64_t shots) {
-    return blog == 5 && n >= 10 && n <= kDenseMaxQubits && shots >= (1ull << n) / 4;
+    return blog == 5 && n >= 10 && n <= kDenseMaxQubits && shots >= kDenseMinShots && shots >= (1ull << n) / 12;
 }
 
 template <typename V, bool PERM>

@@ -95,8 +95,27 @@ def test_many_shots_far_from_unit_norm(scale):
     try:
         S.sv_load_state(h, scale * W.random_state(n, 5))
         cdf = _cdf(h)
-        u = W.uniforms(4 << n, 6)
+        u = W.uniforms(1 << 16, 6)
         # (the rule and its restatement add 2^n FP64 terms in different orders)
         compare_samples(S.sv_sample_uniforms(h, u), u, cdf, cdf[-1] * 2.0 ** (n - 52))
+    finally:
+        S.sv_free(h)
+
+
+@pytest.mark.parametrize("dtype", [S.C64, S.C128])
+@pytest.mark.parametrize("n,shots", [(10, 2 ** 15 - 1), (10, 2 ** 15), (10, 2 ** 15 + 3), (12, 40001), (16, 2 ** 15), (18, 2 ** 15),
+                                     (19, 2 ** 19 // 12 - 1), (19, 2 ** 19 // 12), (19, 2 ** 19 // 12 + 2)])
+@pytest.mark.parametrize("relabel", [0, 1])
+def test_table_line(dtype, n, shots, relabel):
+    """Both sides of the shot counts at which the CDF table takes over."""
+    h = S.sv_alloc(n, dtype)
+    try:
+        S.sv_init_basis(h, 0)
+        S.sv_apply_circuit(h, np.concatenate([W.random_u3_cx(n, 2, 5), W.qft(n)]), relabel=relabel)
+        assert (S.sv_qubit_map(h) != list(range(n))) == bool(relabel)
+        cdf = _cdf(h)
+        u = W.uniforms(shots, 9)
+        u[:2] = 0.0, 1.0 - 2.0 ** -53
+        compare_samples(S.sv_sample_uniforms(h, u), u, cdf, BAND)
     finally:
         S.sv_free(h)
