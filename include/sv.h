@@ -98,8 +98,7 @@ typedef enum {
  * cost-model planner may choose either).
  * pass_kernel: 0 = default (passes run register-resident where they can:
  * every thread keeps 2^5 (c64) / 2^4 (c128) amplitudes of the tile in
- * registers, half as many in plans of default k_max and tile_m that the
- * interpreting kernel runs on up to 20 / 18 qubits, with narrower tiles; tiles move by 16-byte cp.async copies, or, in compiled passes
+ * registers; tiles move by 16-byte cp.async copies, or, in compiled passes
  * whose first / last register layout has coalesced warp accesses, straight
  * between the state and registers), 1 = always the
  * shared-memory pass kernel, 2 = register-resident passes whose tiles move by
@@ -118,6 +117,10 @@ typedef enum {
  * angles from a Walsh-Hadamard transform, and up to five such targets share
  * one pass over the state; exact up to rounding.  0 = runs of at least 64
  * gates, 1 = runs of at least 4 gates, -1 = off.  At most 16 controls.
+ * Small states: with k_max = tile_m = 0 (or the widths sv_last_plan reports),
+ * pass_kernel = 0, CUDA cores and passes that are not compiled, states of up to
+ * 20 (c64) / 18 (c128) qubits take narrower tiles whose threads keep half as
+ * many amplitudes, and states of up to 9 / 8 qubits blocks of 3 / 2 qubits.
  * jit: register-resident passes as kernels compiled at run time (NVRTC) for
  * their structure -- op sequence, gate positions, table masks and register
  * layouts fixed in the code, the data still read from the plan -- and cached
@@ -319,7 +322,10 @@ int sv_expect_z_device(sv_handle h, double *dev_out);
  * Philox4x64-10 (Salmon et al. SC'11): shot s uses word s mod 4 of block
  * Philox(counter = (s div 4, 0, 0, 0), key = (seed, 0)), u = (w >> 11) 2^-53.
  * sv_sample_uniforms takes the uniforms u[0..shots) from the caller (host).
- * Outcomes are uint64 indices, to host or device memory. */
+ * Outcomes are uint64 indices, to host or device memory.  From 2^15 shots and
+ * 2^n / 12 of them on (10 <= n <= 24) the samplers build a table of C, 12 bytes
+ * per amplitude of device memory, which the handle keeps for later calls until
+ * sv_free; without memory for it they do without. */
 int sv_sample(sv_handle h, uint64_t shots, uint64_t seed, uint64_t *host_out);
 int sv_sample_device(sv_handle h, uint64_t shots, uint64_t seed, uint64_t *dev_out);
 int sv_sample_uniforms(sv_handle h, const double *host_u, uint64_t shots, uint64_t *host_out);

@@ -313,7 +313,7 @@ extern "C" int sv_batch_run(int C, const int* n_qubits, const int64_t* gate_offs
         if (po.rb != reg_bits(dt)) {
             // the wave kernel holds the wide register count: a wave has warps
             // enough, and fewer passes and remaps (256 20-qubit ansatz circuits:
-            // 62.9 ms, with 2^4 amplitudes per thread 67.8 ms)
+            // 2^4 amplitudes per thread took 67.8 ms where these took 62.9, now 61.7)
             po.rb = reg_bits(dt);
             po.k_max = dt == SV_C64 ? kMaxK : 4;
             po.tile_m = std::min(n, po.rb + 8);

@@ -241,7 +241,7 @@ __device__ __forceinline__ void reg_swap(V* v) {
 
 // Entries j and j + 1 of a table (complex64: one 16-byte access, tables start on
 // 16 bytes and j is even), held in registers: as operands left in the constant
-// bank they took the compiler two to four times as long per pass.
+// bank they took the compiler four to six times as long per pass.
 template <typename V> __device__ __forceinline__ void hold(V& a) {
     if constexpr (sizeof(V) == 8) asm volatile("" : "+f"(a.x), "+f"(a.y));
 }
