@@ -125,7 +125,7 @@ __host__ __device__ inline int tc_kmajor_index(int n, int kk, int K) {
 }
 
 struct PassDev {
-    double scale;        // register passes: factor applied at write-back (1 unless GR_H records)
+    double scale;        // register passes: factor applied at write-back (1 without deferred factors)
     int n;               // qubits of the state the pass runs on
     int m;
     int L;
@@ -135,6 +135,7 @@ struct PassDev {
     int rb;              // register passes: 2^rb amplitudes per thread
     int folded;          // register passes: some write mask is not the layout's own
     int fmask[kMaxK];    // register passes: the write masks (RemapDev) of the final write-back
+    int angled;          // register passes: the factor depends on angles (it holds rotations')
     int ndiag;           // register passes: diagonal runs (each folded once per tile)
     int nops;            // ops in the pass's region
     int region_off;      // byte offset of the region in the blob

@@ -1887,6 +1887,7 @@ bool reg_region(const Plan& p, const HostPass& hp, PassDev* P, const int* loc, s
                             data.push_back(cd(-tn, -tn));
                         }
                         scale *= c;
+                        P->angled = 1;
                         ++deferred;
                     } else if (gm) {
                         t.off = (int)data.size();
@@ -1944,27 +1945,32 @@ bool register_pass_eligible(const Plan& p, const HostPass& hp) {
 }
 
 // The factors a plan's register passes multiply their amplitudes by become
-// powers of two, exact in every type, in all passes but the last, which takes
-// what remains: one rounding per amplitude, not one per pass.  (Passes are
-// linear: the state between two of them may be off by a factor of up to
-// sqrt(2).  Tensor-core passes restore their own norm and keep their factor.)
+// powers of two, exact in every type, in all passes but one, which takes what
+// remains of those before it: one rounding per amplitude, not one per pass.
+// It is the last pass with rotations, as compiled code holds the factors of the
+// others as constants and must not change with the angles.  (Passes are linear:
+// the state between two of them may be off by a factor of up to 1.5.
+// Tensor-core passes restore their own norm and keep their factor.)
 static void gather_factors(PassDev* pd, size_t count) {
     auto has = [](const PassDev& P) { return (P.rmode == 1 || P.rmode == 2) && P.tc_k == 0 && P.scale != 1.0; };
+    bool angles = false;
+    for (size_t i = 0; i < count; ++i) angles |= has(pd[i]) && pd[i].angled;
     size_t last = count;
     for (size_t i = 0; i < count; ++i)
-        if (has(pd[i])) last = i;
+        if (has(pd[i]) && (pd[i].angled || !angles)) last = i;
     double rest = 1.0;
     for (size_t i = 0; i < count && last < count; ++i) {
         if (!has(pd[i])) continue;
-        const double t = pd[i].scale * rest;
         if (i == last) {
-            pd[i].scale = t;
+            pd[i].scale *= rest;
             break;
         }
+        const bool own = angles && !pd[i].angled;  // (Hadamards': a constant of the pass)
+        const double t = own ? pd[i].scale : pd[i].scale * rest;
         int e;
         const double m = std::frexp(std::fabs(t), &e);  // in [1/2, 1)
-        pd[i].scale = std::copysign(std::ldexp(m < 0.70710678 ? 0.5 : 1.0, e), t);
-        rest = t / pd[i].scale;
+        pd[i].scale = std::copysign(std::ldexp(m < 0.75 ? 0.5 : 1.0, e), t);
+        rest = own ? rest * (t / pd[i].scale) : t / pd[i].scale;
     }
 }
 

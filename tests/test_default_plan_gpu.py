@@ -165,3 +165,22 @@ def test_many_passes_round_their_factor_once():
         for what, opts in (("small", {}), ("wide", dict(k_max=5, tile_m=13))):
             err[what].append(np.linalg.norm(U.run_gpu(n, g, S.C64, **opts) - ref))
     assert np.mean(err["small"]) <= 1.04 * np.mean(err["wide"])
+
+
+def test_new_angles_reuse_compiled_hadamard_passes():
+    """A pass that holds Hadamards only (the second of these plans) keeps its
+    compiled code when the angles of the one before it change."""
+    n = 14
+    before = None
+    for seed in range(3):
+        a = np.random.default_rng(seed).uniform(0.2, 2.8, size=(2, 13))
+        items = [(W.RY, (q,), (float(a[0, q]),)) for q in range(13)] + [(W.CX, (q, (q + 1) % 13), ()) for q in range(13)]
+        items += [(W.RY, (q,), (float(a[1, q]),)) for q in range(13)]
+        items += [(W.H, (13,), ()), (W.CX, (13, 0), ()), (W.H, (0,), ()), (W.CX, (0, 13), ()), (W.H, (13,), ())]
+        g = W.gates_from_list(items)
+        second = [op for op in S.sv_plan_ops(n, S.C64, g, k_max=5, tile_m=13) if op["pass"] == 1]
+        assert [list(op["qubits"]) for op in second] == [[0, 13]]
+        U.assert_close(U.run_gpu(n, g, S.C64, jit=1), U.run_oracle(n, g), S.C64, "seed %d" % seed)
+        if seed:
+            assert S.sv_jit_stats()["compiled"] == before
+        before = S.sv_jit_stats()["compiled"]
