@@ -51,16 +51,16 @@ UNIT = "amp_updates/s"
 
 # DRAM traffic of the tile pass per amplitude per launch, from the ncu capture
 # summarised in profiles/ (the bench's random U3+CX family at n=26 complex64,
-# the 85 passes of one step on the run-time compiled kernels;
+# the 64 passes of one step on the run-time compiled kernels;
 # dram__bytes_read.sum + dram__bytes_write.sum), valid only for the kernel,
 # compiler and planner sources it was taken with (SHA-256 over the files
 # below); a changed kernel reports traffic null until it is captured again.
 TRAFFIC_SOURCES = ["paper_2504_03967_gb300/csrc/sv_apply.cu", "paper_2504_03967_gb300/csrc/sv_plan.cpp",
                    "paper_2504_03967_gb300/csrc/sv_internal.h", "paper_2504_03967_gb300/csrc/sv_dev.h",
                    "paper_2504_03967_gb300/csrc/sv_rpass.cuh", "paper_2504_03967_gb300/csrc/sv_jit.cpp"]
-TRAFFIC = {"sha256": "4bd6035baccc91a93d8298223b5a143c53015278da0dbc1a6127ae6bba04ed82",
-           "bytes_per_amp": 15.398,
-           "profile": "profiles/traffic_random26_c64_bench.md (the 85 tile passes of one step at n=26, scaled to 2^n)"}
+TRAFFIC = {"sha256": "43e244064f967c21b901b10bd0fc1cc62944f22351cb983883a344e244be9a5f",
+           "bytes_per_amp": 15.149,
+           "profile": "profiles/traffic_random26_c64_bench.md (the 64 tile passes of one step at n=26, scaled to 2^n)"}
 
 
 def sources_sha(read=None):
